@@ -56,6 +56,7 @@ struct Workspace {
   unsigned* gbar = nullptr;                                // grid barrier state (count, gen)
   int coop_blocks = 0;                                     // 0: fused kernel not usable
   int units_blocks = 0;                                    // grid of the multi-RHS fused kernel
+  bool run_ok = false;                                     // one RHS: whole runs by k_gmres_run
   double2 *pblk = nullptr, *hred = nullptr;                // fused kernel: block partials, totals
   int arn_smem = 0;                                        // fused kernel: dynamic shared bytes
   double2* pbu = nullptr;                                  // multi-RHS fused kernel: unit partials
@@ -1867,7 +1868,55 @@ __global__ void k_pad_copy(const float2* __restrict__ src, int n, int ld, int nr
   dst[i] = r < n ? src[(size_t)s * n + r] : make_float2(0.f, 0.f);
 }
 
+}  // namespace natbem
+
+#include "gmres_run.cuh"
+
+namespace natbem {
+
 // ---------------------------------------------------------------------------- host side
+// The kernel of a whole run (gmres_run.cuh) for the operator's format and the basis' precision.
+static const void* run_kernel(int fmt, bool f32) {
+  switch (fmt) {
+    case 0: return (const void*)k_gmres_run<0, false>;
+    case 1: return f32 ? (const void*)k_gmres_run<1, true> : (const void*)k_gmres_run<1, false>;
+    default: return f32 ? (const void*)k_gmres_run<2, true> : (const void*)k_gmres_run<2, false>;
+  }
+}
+
+// Shape of k_gmres_run for an operator of `n` rows (stages = 0: it does not fit) and its grid:
+// one block per SM, at least eight rows a block.
+static RunArgs run_fit(int n, int ld, int blocks, int fmt, bool f32, int cols, int* grid) {
+  *grid = std::max(1, std::min(blocks, (n + 7) / 8));
+  return run_shape(n, ld, *grid, fmt, f32, cols);
+}
+
+// Whether every form of the kernel is launchable on the current device.
+static bool run_usable() {
+  static std::mutex mu;
+  static int ready[64] = {0};
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (dev < 0 || dev >= 64) return false;
+  {
+    std::lock_guard<std::mutex> lk(mu);
+    if (ready[dev] == 0) {
+      ready[dev] = 1;
+      for (int f = 0; f < 3; ++f)
+        for (int b = 0; b < 2; ++b) {
+          int per_sm = 0;
+          if (cudaFuncSetAttribute(run_kernel(f, b), cudaFuncAttributeMaxDynamicSharedMemorySize, kRunSmem) != cudaSuccess ||
+              cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, run_kernel(f, b), kRunThreads, kRunSmem) != cudaSuccess ||
+              per_sm < 1) {
+            cudaGetLastError();
+            ready[dev] = -1;
+          }
+        }
+    }
+    return ready[dev] > 0;
+  }
+}
+
 // Krylov dimension: the restart length of GMRES(m), or the iteration cap when unrestarted.
 static int krylov_dim(const nat_bem_opts& o) {
   const int cap = std::max(1, o.max_iter);
@@ -2024,6 +2073,7 @@ static nat_bem_status workspace_ensure(nat_bem_op* op, int nrhs, cudaStream_t s)
         NB_TRY(dev_alloc_n(&ws->pbu, most * (mm + 2), s));
       }
       NB_TRY(dev_alloc_n(&ws->wf, (size_t)n * nr, s));  // FP32 w of inner solves on the FP32 basis
+      ws->run_ok = nrhs == 1 && op->bstride == 0 && !std::getenv("NATBEM_NO_RUN_KERNEL") && run_usable();
     }
   }
   NB_TRY_CUDA(cudaMemsetAsync(ws->tc_err, 0, sizeof(int), s));
@@ -2405,6 +2455,33 @@ static void loop_count(Workspace* ws) {
 static nat_bem_status gmres_run(nat_bem_op* op, Workspace* ws, const GArgs& a, int engine,
                                 int accumulate, float2* pout, cudaStream_t s) {
   const int n = (int)op->n, nrhs = ws->nrhs;
+  // One right-hand side: the whole run in one cooperative launch where the block's share of the
+  // operator's rows fits its registers and shared memory, up to about 10,000 rows of complex64 and
+  // 12,000 of a 16-bit copy (per-launch tracing keeps the two-launch iteration, whose kernels it
+  // times). Measured with one solve in flight, two-launch form -> this, a whole solve: 1280 rows
+  // FP32 1037 -> 478 us, 3956 783 -> 466, 5174 1888 -> 1401, 10240 5878 -> 4299; 10240 mixed BF16
+  // 4283 -> 3643. Above that the matvec streams for 10x the time of the rest of an iteration.
+  if (ws->run_ok && nrhs == 1 && op->bstride == 0 && !tracing_enabled()) {
+    const int fmt = engine == kEngineGemv ? 0 : (op->copy_fp16 ? 2 : 1);
+    int grid = 0;
+    RunArgs r = run_fit(n, (int)ws->ld, ws->coop_blocks, fmt, a.Vf != nullptr, a.maxit + 1, &grid);
+    if (r.stages > 0) {
+      r.A = fmt == 0 ? (const void*)op->L : (const void*)op->Lb;
+      r.rs = fmt == 2 ? op->row_scale : nullptr;
+      r.pb = ws->pblk;
+      r.hr = ws->hred;
+      r.bar = ws->gbar;
+      r.err = ws->tc_err;
+      r.pout = pout;
+      r.accumulate = accumulate;
+      GArgs ac = a;
+      void* args[] = {&ac, &r};
+      NB_LAUNCH("gmres_run", s, NB_TRY_CUDA(cudaLaunchCooperativeKernel(run_kernel(fmt, a.Vf != nullptr), dim3(grid),
+                                                                       dim3(kRunThreads), args, (size_t)kRunSmem, s)));
+      NB_CHECK_LAUNCH();
+      return NAT_BEM_OK;
+    }
+  }
   const dim3 upd_grid(ws->nchunk, nrhs), fin_grid((n + kChunk - 1) / kChunk, nrhs);
   // the dot-product grid covers the Krylov vectors 0..j of the iteration being launched (the
   // device's j equals the host's launch count until every RHS is done)
@@ -2732,6 +2809,10 @@ nat_bem_status solve_impl(nat_bem_op* op, const float2* d_neumann, int nrhs, flo
       loop_copy(ws, s);
       NB_TRY_CUDA(cudaStreamSynchronize(s));  // one host sync per sweep
       loop_count(ws);
+      if (tc_err) {
+        set_error("GMRES: a bounded wait gave up (code " + std::to_string(tc_err) + ")");
+        return NAT_BEM_ECUDA;
+      }
       int used = 0;
       for (int q = 0; q < nrhs; ++q) {
         total[q] += iters[q];
