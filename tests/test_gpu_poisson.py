@@ -113,3 +113,25 @@ def test_device_tensors(nb):
     assert np.array_equal(idx, ai)
     assert np.array_equal(x.cpu().numpy(), ax)
     assert np.array_equal(n.cpu().numpy(), an)
+
+
+def test_long_candidate_lists(nb):
+    """Cells with more candidates than a warp has lanes, in one and in several phases."""
+    V, F = S.icosphere(2)
+    _check(nb, V, F, np.random.default_rng(8).random((6000, 3)), 0.45)
+    _check(nb, V, F, np.random.default_rng(9).random((3000, 3)), 1.1)
+
+
+@pytest.mark.parametrize("scale,shift", [(1.0, 0.0), (1e-9, 0.0), (1.0, 1e6), (1e9, -3e10)])
+def test_distances_at_the_radius(nb, scale, shift):
+    """Radii equal to a distance between two candidates, and one unit in the last place to either
+    side: the FP32 screen has to leave these to the FP64 test, at any scale and offset."""
+    V, F = S.icosphere(2)
+    V = V * scale + shift
+    u = np.random.default_rng(10).random((600, 3))
+    x, _, _ = P.candidates(V, F, u)
+    d = x[1:] - x[0]
+    d = np.sqrt((d[:, 0] * d[:, 0] + d[:, 1] * d[:, 1]) + d[:, 2] * d[:, 2])
+    for r in np.sort(d)[[5, 40, 120]]:
+        for q in (r, np.nextafter(r, 0.0), np.nextafter(r, 1e300)):
+            _check(nb, V, F, u, float(q))
