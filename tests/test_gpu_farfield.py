@@ -122,3 +122,25 @@ def test_dataset_step_at_full_size(nb, oracle_lib):
     dpick = np.random.default_rng(72).choice(len(dirs), 48, replace=False)
     ref_ff = oracle_lib.far_field(V, F, k, dirs[dpick], p64, g64)
     assert _rel(ff[dpick], ref_ff) < TOL
+
+
+# Random surface data: the sum over 302 x 7 terms cancels to its root mean square, so FP32 terms
+# (a few 6e-8 each, phases up to k r = 18 rounded at 1e-6) leave at most about 1e-6 x sqrt(N / N_eff)
+# ~ 5e-6 of the result; 2e-5 holds for every pass width and remainder.
+@pytest.mark.parametrize("nrhs", [1, 2, 3, 4, 5, 9, 17, 33])
+@pytest.mark.parametrize("n_tri,m", [(8, 1), (302, 127), (1218, 129)])
+def test_field_and_far_field_pass_widths_and_remainders(nb, oracle_lib, n_tri, m, nrhs):
+    Vs, F = S.ring_sphere(n_tri)
+    V = S.perturbed_ellipsoid(Vs, 41) + np.array([3.0, -1.0, 0.5])
+    k = 2.37
+    rng = np.random.default_rng(n_tri + nrhs)
+    p, g = ((rng.normal(size=(n_tri, nrhs)) + 1j * rng.normal(size=(n_tri, nrhs))).astype(np.complex64) for _ in range(2))
+    pts = S.shell_points(m, 6.0, 9.0, 3)
+    dirs = S.fibonacci_points(m, 1.0) if m > 1 else np.array([[0.0, 0.6, 0.8]])
+    with nb.Operator.assemble(V, F, k) as op:
+        f, far = op.evaluate(pts, p, g), op.far_field(dirs, p, g)
+    for s in (0, nrhs - 1):
+        ref = oracle_lib.evaluate(V, F, k, pts, p[:, s], g[:, s])
+        assert _rel(f[:, s], ref) < 2e-5
+        ref = oracle_lib.far_field(V, F, k, dirs, p[:, s], g[:, s])
+        assert _rel(far[:, s], ref) < 2e-5
