@@ -12,7 +12,8 @@
 // scratch arrays of pair blocks. The gathers then sum, for every vertex i and column (vertex j,
 // or triangle s), the blocks of the triangles around i (and around j) in a fixed order, so the
 // result does not depend on scheduling: k_gal_rowsum_L first sums each test triangle's row over
-// the triangles around every column vertex (reading each pair block once), k_gal_gather_L and
+// the triangles around every column vertex (reading each pair block once; from planes over the
+// trial triangle 338 us at 5120 triangles, from 72-byte blocks 556), k_gal_gather_L and
 // k_gal_gather_R then sum over the triangles around each row vertex. FP32 arithmetic throughout: near the
 // singularity x - y is formed from the transformed coordinates (a radius times a bounded
 // vector), and for regular pairs from the centroid difference (hi/lo pairs) plus the points'
@@ -26,6 +27,7 @@
 #include <vector>
 
 #include "internal.h"
+#include "pairs.cuh"
 
 namespace natbem {
 
@@ -33,9 +35,6 @@ namespace {
 constexpr int kGalSing = 4;          // Gauss-Legendre points per dimension on singular pairs
 constexpr int kGalVals = 12;         // per pair: L block (a, b) at 3a + b, then R entries (a)
 constexpr double kGalScratch = 4e9;  // bytes of pair blocks per round of test triangles
-constexpr float kTwoPiHi = 6.28318548202514648f;
-constexpr float kTwoPiLo = -1.7484555314695172e-7f;
-constexpr float kInvTwoPi = 0.159154943091895336f;
 constexpr float kInv4Pi = 0.0795774715459476679f;
 constexpr float kFourPi = 12.5663706143591730f;
 
@@ -47,127 +46,81 @@ __device__ __forceinline__ uint32_t gal_pack_bf16(float re, float im) {
   return *reinterpret_cast<uint32_t*>(&v);
 }
 
-// Weighted kernels at x - y = d: w G, w dG/dn_y, w dG/dn_x (w includes 1 / (4 pi)).
-struct GalK {
-  float gr, gi, yr, yi, xr, xi;
-};
-
-// dny = d . n_y and dnx = d . n_x, given by the caller.
-__device__ __forceinline__ GalK gal_kernels_dn(float dx, float dy, float dz, float k, float w, float dny,
-                                               float dnx) {
-  const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-  const float rinv = rsqrtf(r2);
-  const float rho = k * (r2 * rinv);
-  const float nq = rintf(rho * kInvTwoPi);
-  float th = fmaf(-nq, kTwoPiHi, rho);
-  th = fmaf(-nq, kTwoPiLo, th);
-  float sn, cs;
-  __sincosf(th, &sn, &cs);
-  const float gw = rinv * w;
-  GalK o;
-  o.gr = cs * gw;
-  o.gi = sn * gw;
-  const float r2inv = rinv * rinv;
-  const float fr = fmaf(rho, o.gi, o.gr) * r2inv, fi = fmaf(-rho, o.gr, o.gi) * r2inv;
-  o.yr = fr * dny;
-  o.yi = fi * dny;
-  o.xr = -fr * dnx;
-  o.xi = -fi * dnx;
-  return o;
-}
-
-__device__ __forceinline__ GalK gal_kernels(float dx, float dy, float dz, float k, float w, float3 nx,
-                                            float3 ny) {
-  const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-  const float rinv = rsqrtf(r2);
-  const float rho = k * (r2 * rinv);
-  const float nq = rintf(rho * kInvTwoPi);
-  float th = fmaf(-nq, kTwoPiHi, rho);
-  th = fmaf(-nq, kTwoPiLo, th);
-  float sn, cs;
-  __sincosf(th, &sn, &cs);
-  const float gw = rinv * w;
-  GalK o;
-  o.gr = cs * gw;
-  o.gi = sn * gw;
-  // G (1 - i rho) / r^2, times d.n_y (dG/dn_y) and -d.n_x (dG/dn_x)
-  const float r2inv = rinv * rinv;
-  const float fr = fmaf(rho, o.gi, o.gr) * r2inv, fi = fmaf(-rho, o.gr, o.gi) * r2inv;
-  const float dny = fmaf(dx, ny.x, fmaf(dy, ny.y, dz * ny.z));
-  const float dnx = fmaf(dx, nx.x, fmaf(dy, nx.y, dz * nx.z));
-  o.yr = fr * dny;
-  o.yi = fi * dny;
-  o.xr = -fr * dnx;
-  o.xi = -fi * dnx;
-  return o;
-}
-
-// Per-pair sums: Kb[a][b] = sum w lam_a mu_b dG/dn_y, Gb[a][b] = sum w lam_a mu_b G,
-// Kp[a] = sum w lam_a dG/dn_x (complex, interleaved re/im).
+// Per-pair sums over x in tau, y in sigma, d = x - y, with F = G (1 - i k r) / r^2:
+// gb[a][b] = sum w lam_a mu_b G, ky[a][b] = sum w lam_a mu_b F d.n_sigma, kx[a][b] = sum w lam_a mu_b F d.n_tau
+// (complex, interleaved). dG/dn_y = F d.n_sigma and dG/dn_x = -F d.n_tau, and with the roles
+// swapped d changes sign: the three sums give the blocks of both (tau, sigma) and (sigma, tau).
 struct GalAcc {
-  float kb[18], gb[18], kp[6];
+  float gb[18], ky[18], kx[18];
 };
 
 __device__ __forceinline__ void gal_acc_zero(GalAcc& A) {
 #pragma unroll
-  for (int i = 0; i < 18; ++i) A.kb[i] = A.gb[i] = 0.f;
-#pragma unroll
-  for (int i = 0; i < 6; ++i) A.kp[i] = 0.f;
+  for (int i = 0; i < 18; ++i) A.gb[i] = A.ky[i] = A.kx[i] = 0.f;
 }
 
-__device__ __forceinline__ void gal_acc_point(GalAcc& A, const float (&lam)[3], const float (&mu)[3],
-                                              const GalK& v) {
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-      const float lm = lam[a] * mu[b];
-      A.kb[2 * (3 * a + b)] = fmaf(lm, v.yr, A.kb[2 * (3 * a + b)]);
-      A.kb[2 * (3 * a + b) + 1] = fmaf(lm, v.yi, A.kb[2 * (3 * a + b) + 1]);
-      A.gb[2 * (3 * a + b)] = fmaf(lm, v.gr, A.gb[2 * (3 * a + b)]);
-      A.gb[2 * (3 * a + b) + 1] = fmaf(lm, v.gi, A.gb[2 * (3 * a + b) + 1]);
-    }
-    A.kp[2 * a] = fmaf(lam[a], v.xr, A.kp[2 * a]);
-    A.kp[2 * a + 1] = fmaf(lam[a], v.xi, A.kp[2 * a + 1]);
-  }
+// w G and w F (w includes 1 / (4 pi)); turns: the phase's nearest number of turns, or a
+// nearby point's.
+__device__ __forceinline__ void gal_kernels(float rinv, float rho, float turns, float w, float2& G, float2& F) {
+  float th = fmaf(-turns, kTwoPiHi, rho);
+  th = fmaf(-turns, kTwoPiLo, th);
+  float sn, cs;
+  __sincosf(th, &sn, &cs);
+  const float gw = rinv * w;
+  G.x = cs * gw;
+  G.y = sn * gw;
+  const float r2inv = rinv * rinv;
+  F.x = fmaf(rho, G.y, G.x) * r2inv;
+  F.y = fmaf(-rho, G.x, G.y) * r2inv;
 }
+__device__ __forceinline__ float gal_turns(float rho) { return fmaf(rho, kInvTwoPi, kRound) - kRound; }
 
-// The pair's 12 values: L block -Kb - beta H and R entries -Vb - beta Kp (beta = i / k), with
-// H = k^2 (n_t . n_s) Gb - (curl_a^t . curl_b^s) G0, Vb[a] = sum_b Gb[a][b], G0 = sum Gb.
+// The 12 values of (tau, sigma), or with kSwap of (sigma, tau): L block -Kb - beta H and R entries
+// -Vb - beta Kp (beta = i / k), with H = k^2 (n_t . n_s) Gb - (curl_a^t . curl_b^s) G0,
+// Vb[a] = sum_b Gb[a][b], G0 = sum Gb, Kp[a] the sum of dG/dn_x over the trial triangle.
+template <bool kSwap>
 __device__ __forceinline__ void gal_finish(const GalAcc& A, float k, float nn, const float (&cc)[9],
                                            float2 (&out)[kGalVals]) {
-  const float kinv = 1.f / k, k2 = k * k;
+  const float kinv = 1.f / k, k2nn = k * k * nn;
   float g0r = 0.f, g0i = 0.f;
 #pragma unroll
   for (int i = 0; i < 9; ++i) {
     g0r += A.gb[2 * i];
     g0i += A.gb[2 * i + 1];
   }
-#pragma unroll
-  for (int i = 0; i < 9; ++i) {
-    const float hr = k2 * nn * A.gb[2 * i] - cc[i] * g0r;
-    const float hi = k2 * nn * A.gb[2 * i + 1] - cc[i] * g0i;
-    // -Kb - (i/k) H = (-Kb_r + H_i / k, -Kb_i - H_r / k)
-    out[i] = make_float2(-A.kb[2 * i] + hi * kinv, -A.kb[2 * i + 1] - hr * kinv);
-  }
+  const float* kb = kSwap ? A.kx : A.ky;  // dG/dn_y, up to the sign of d
+  const float* kp = kSwap ? A.ky : A.kx;  // -dG/dn_x, likewise
+  const float sg = kSwap ? -1.f : 1.f;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    const float vr = A.gb[2 * (3 * a)] + A.gb[2 * (3 * a + 1)] + A.gb[2 * (3 * a + 2)];
-    const float vi = A.gb[2 * (3 * a) + 1] + A.gb[2 * (3 * a + 1) + 1] + A.gb[2 * (3 * a + 2) + 1];
-    out[9 + a] = make_float2(-vr + A.kp[2 * a + 1] * kinv, -vi - A.kp[2 * a] * kinv);
+    float vr = 0.f, vi = 0.f, pr = 0.f, pi = 0.f;
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      const int i = kSwap ? 3 * b + a : 3 * a + b;
+      const float hr = k2nn * A.gb[2 * i] - cc[i] * g0r;
+      const float hi = k2nn * A.gb[2 * i + 1] - cc[i] * g0i;
+      // -Kb - (i/k) H = (-Kb_r + H_i / k, -Kb_i - H_r / k)
+      out[3 * a + b] = make_float2(-sg * kb[2 * i] + hi * kinv, -sg * kb[2 * i + 1] - hr * kinv);
+      vr += A.gb[2 * i];
+      vi += A.gb[2 * i + 1];
+      pr -= sg * kp[2 * i];
+      pi -= sg * kp[2 * i + 1];
+    }
+    out[9 + a] = make_float2(-vr + pi * kinv, -vi - pr * kinv);
   }
 }
 
-// Pair (t, s) of the round starting at t0: the L block at partL[((t - t0) nt + s) 9 + 3a + b],
-// the R entries at partR[((t - t0) 3 + a) nt + s] (contiguous over s for the R gather).
+// Pair blocks of a round: value i of pair (t, s), i < 9 the L block at 3a + b, then the R entries,
+// in planes over s: partL[((t - t0) 9 + i) nt + s], partR[((t - t0) 3 + a) nt + s].
+__device__ __forceinline__ float2* gal_plane(float2* partL, float2* partR, int nt, int tr, int i) {
+  return i < 9 ? partL + ((size_t)tr * 9 + i) * nt : partR + ((size_t)tr * 3 + i - 9) * nt;
+}
 __device__ __forceinline__ void gal_store(float2* partL, float2* partR, int nt, int tr, int s,
                                           const float2 (&v)[kGalVals]) {
-  float2* pl = partL + ((size_t)tr * nt + s) * 9;
 #pragma unroll
-  for (int i = 0; i < 9; ++i) pl[i] = v[i];
-#pragma unroll
-  for (int a = 0; a < 3; ++a) partR[((size_t)tr * 3 + a) * nt + s] = v[9 + a];
+  for (int i = 0; i < kGalVals; ++i) gal_plane(partL, partR, nt, tr, i)[s] = v[i];
 }
+constexpr int kGalT = 8;  // test triangles of a block of k_gal_regular (a warp each)
 }  // namespace
 
 // Per element: the three P1 curls (P_{a+1} - P_{a+2}) / (2A); per quadrature point (7 per
@@ -201,14 +154,26 @@ __global__ void k_gal_geometry(const double* __restrict__ tri, const double* __r
   }
 }
 
-// Pairs sharing no vertex: block row tau = t0 + blockIdx.y, one thread per trial triangle.
-__global__ void __launch_bounds__(256, 2)
+// Pairs sharing no vertex: a block has eight test triangles t, a warp each, and 32 triangles s, a
+// lane each. A thread computes (t, s) and (s, t) together where both rows belong to the round: s > t
+// then, and those with t0 <= s <= t are left out. For a flat sigma d.n_sigma depends on x alone, and
+// d.n_tau on y alone, so both normal derivatives come from the sums of F. The blocks (s, t) go
+// through shared memory, so both directions are stored in runs (256 and 64 bytes).
+//
+// Bound by the FMA pipe: about 2300 operations for the two blocks (2 x 2310 when every ordered pair
+// was formed by itself, with the projections in the innermost loop); 5120 triangles: 2.71 ms
+// before, 1.34 ms now (1.67 with the blocks (s, t) stored by each thread in 72-byte pieces).
+__global__ void __launch_bounds__(kGalT * 32, 2)
 k_gal_regular(const float4* __restrict__ c_hi, const float4* __restrict__ c_lo, const float4* __restrict__ nrm,
               const float4* __restrict__ qp, const int4* __restrict__ vid, const float4* __restrict__ curl,
-              int nt, int t0, float k, float2* __restrict__ partL, float2* __restrict__ partR) {
-  const int t = t0 + blockIdx.y;
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= nt) return;
+              int nt, int t0, int t1, float k, float2* __restrict__ partL, float2* __restrict__ partR) {
+  __shared__ float2 s_st[kGalVals][32][kGalT + 1];
+  __shared__ unsigned s_ok[kGalT];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int tb = t0 + blockIdx.y * kGalT, sb0 = blockIdx.x * 32;
+  if (sb0 >= t0 && sb0 + 31 <= tb) return;  // every pair of the tile is another tile's
+  const int t = min(tb + w, t1 - 1), s = min(sb0 + lane, nt - 1);
+  bool live = tb + w < t1 && sb0 + lane < nt && !(s >= t0 && s <= t);
   const int4 vt = vid[t], vs = vid[s];
   const int va[3] = {vt.x, vt.y, vt.z}, vb[3] = {vs.x, vs.y, vs.z};
   bool touch = false;
@@ -216,84 +181,100 @@ k_gal_regular(const float4* __restrict__ c_hi, const float4* __restrict__ c_lo, 
   for (int a = 0; a < 3; ++a)
 #pragma unroll
     for (int b = 0; b < 3; ++b) touch |= va[a] == vb[b];
-  if (touch) return;  // k_gal_singular writes this pair
+  live = live && !touch;  // k_gal_singular writes the pairs that touch
+  const bool both = live && s >= t0 && s < t1;
+  const unsigned oks = __ballot_sync(0xffffffffu, both);
+  if (lane == 0) s_ok[w] = oks;
+  if (live) {
   const float4 th = c_hi[t], tl = c_lo[t], sh = c_hi[s], sl = c_lo[s];
   const float Dx = (th.x - sh.x) + (tl.x - sl.x);
   const float Dy = (th.y - sh.y) + (tl.y - sl.y);
   const float Dz = (th.z - sh.z) + (tl.z - sl.z);
-  const float4 nt4 = nrm[t], ns4 = nrm[s];
-  const float3 nx = make_float3(nt4.x, nt4.y, nt4.z), ny = make_float3(ns4.x, ns4.y, ns4.z);
-  float4 qs[7];
-  float qny[7], qnx[7];  // y_q . n_y and y_q . n_x of the trial points' offsets
+  const float4 nx = nrm[t], ny = nrm[s];
+  const float Dny = fmaf(Dx, ny.x, fmaf(Dy, ny.y, Dz * ny.z)), Dnx = fmaf(Dx, nx.x, fmaf(Dy, nx.y, Dz * nx.z));
+  // trial points: the centroid, then the first orbit's points towards vertices 0, 1, 2 and the
+  // second orbit's at kOrbit times the same offsets
+  float bx[3], by[3], bz[3], nb[3];
+  float wc, wo[2];
 #pragma unroll
-  for (int q = 0; q < 7; ++q) {
-    qs[q] = qp[7 * (size_t)s + q];
-    qny[q] = fmaf(qs[q].x, ny.x, fmaf(qs[q].y, ny.y, qs[q].z * ny.z));
-    qnx[q] = fmaf(qs[q].x, nx.x, fmaf(qs[q].y, nx.y, qs[q].z * nx.z));
+  for (int m = 0; m < 3; ++m) {
+    const float4 q = qp[7 * (size_t)s + 3 - m];
+    bx[m] = q.x;
+    by[m] = q.y;
+    bz[m] = q.z;
+    nb[m] = fmaf(q.x, nx.x, fmaf(q.y, nx.y, q.z * nx.z));
+    wo[0] = q.w;
   }
+  wc = qp[7 * (size_t)s].w;
+  wo[1] = qp[7 * (size_t)s + 4].w;
   GalAcc A;
   gal_acc_zero(A);
 #pragma unroll 1
   for (int p = 0; p < 7; ++p) {
     const float4 qt = qp[7 * (size_t)t + p];
     const float wx = qt.w * kFourPi;  // w_p A_tau (the 1 / (4 pi) is in the trial weights)
-    // x_p - y_q = (D + x_p offset) - y_q offset; its projections likewise
     const float px = Dx + qt.x, py = Dy + qt.y, pz = Dz + qt.z;
-    const float pny = fmaf(px, ny.x, fmaf(py, ny.y, pz * ny.z)), pnx = fmaf(px, nx.x, fmaf(py, nx.y, pz * nx.z));
-    // inner sums over the trial points, then the test basis functions. The rule's points are
-    // the centroid (weights 1/3 on every basis function) and two orbits whose barycentric
-    // coordinates permute (e, e, 1 - 2e): on an orbit, sum_q mu_b(q) v_q = e S + (1 - 3e) v_q*,
-    // S the orbit's sum and q* its point with 1 - 2e on vertex b.
-    float sg[6], sy[6], sx[2];
+    const float pny = Dny + fmaf(qt.x, ny.x, fmaf(qt.y, ny.y, qt.z * ny.z));
+    // inner sums over the trial points per basis function b, of G, F and F d.n_tau. On an orbit
+    // with barycentrics (e, e, 1 - 2e): sum_q mu_b(q) v_q = e S + (1 - 3e) v_b, S the orbit's sum
+    // and v_b its point towards vertex b; the centroid counts a third on every b.
+    float cm[6], sb[3][6];
+    float turns;
     {
-      const GalK v = gal_kernels_dn(px - qs[0].x, py - qs[0].y, pz - qs[0].z, k, qs[0].w, pny - qny[0], pnx - qnx[0]);
+      const float r2 = fmaf(px, px, fmaf(py, py, pz * pz));
+      const float rinv = rsqrtf(r2), rho = k * (r2 * rinv);
+      turns = gal_turns(rho);
+      float2 G, F;
+      gal_kernels(rinv, rho, turns, wc, G, F);
       const float third = c_gal_b7[0][0];
-#pragma unroll
-      for (int b = 0; b < 3; ++b) {
-        sg[2 * b] = third * v.gr;
-        sg[2 * b + 1] = third * v.gi;
-        sy[2 * b] = third * v.yr;
-        sy[2 * b + 1] = third * v.yi;
-      }
-      sx[0] = v.xr;
-      sx[1] = v.xi;
+      cm[0] = third * G.x;
+      cm[1] = third * G.y;
+      cm[2] = third * F.x;
+      cm[3] = third * F.y;
+      cm[4] = cm[2] * Dnx;
+      cm[5] = cm[3] * Dnx;
     }
 #pragma unroll
     for (int o = 0; o < 2; ++o) {
-      const int q0 = 1 + 3 * o;  // points q0, q0 + 1, q0 + 2 carry 1 - 2e on vertex 2, 1, 0
-      float vg[3][4];
+      const float c = o == 0 ? -1.f : -kOrbit;
+      const float e = c_gal_b7[1 + 3 * o][0], f = c_gal_b7[1 + 3 * o][2] - e;  // e and 1 - 3e
+      float S[6];
 #pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        const int q = q0 + i;
-        const GalK v = gal_kernels_dn(px - qs[q].x, py - qs[q].y, pz - qs[q].z, k, qs[q].w, pny - qny[q], pnx - qnx[q]);
-        vg[i][0] = v.gr;
-        vg[i][1] = v.gi;
-        vg[i][2] = v.yr;
-        vg[i][3] = v.yi;
-        sx[0] += v.xr;
-        sx[1] += v.xi;
+      for (int m = 0; m < 3; ++m) {
+        const float dx = fmaf(c, bx[m], px), dy = fmaf(c, by[m], py), dz = fmaf(c, bz[m], pz);
+        const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+        const float rinv = rsqrtf(r2), rho = k * (r2 * rinv);
+        float2 G, F;
+        gal_kernels(rinv, rho, turns, wo[o], G, F);
+        const float dnx = fmaf(c, nb[m], Dnx);
+        const float v[6] = {G.x, G.y, F.x, F.y, F.x * dnx, F.y * dnx};
+#pragma unroll
+        for (int i = 0; i < 6; ++i) {
+          S[i] = m == 0 ? v[i] : S[i] + v[i];
+          sb[m][i] = o == 0 ? f * v[i] : fmaf(f, v[i], sb[m][i]);
+        }
       }
-      const float e = c_gal_b7[q0][0], f = c_gal_b7[q0][2] - e;  // e and 1 - 3e
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const float S = e * ((vg[0][c] + vg[1][c]) + vg[2][c]);
-        float* acc = c < 2 ? sg : sy;
+      for (int i = 0; i < 6; ++i) cm[i] = fmaf(e, S[i], cm[i]);
+    }
 #pragma unroll
-        for (int b = 0; b < 3; ++b) acc[2 * b + (c & 1)] += fmaf(f, vg[2 - b][c], S);
-      }
+    for (int b = 0; b < 3; ++b) {
+#pragma unroll
+      for (int i = 0; i < 6; ++i) sb[b][i] += cm[i];
+      sb[b][2] *= pny;
+      sb[b][3] *= pny;
     }
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
       const float la = c_gal_b7[p][a] * wx;
 #pragma unroll
-      for (int b = 0; b < 3; ++b) {
-        A.kb[2 * (3 * a + b)] = fmaf(la, sy[2 * b], A.kb[2 * (3 * a + b)]);
-        A.kb[2 * (3 * a + b) + 1] = fmaf(la, sy[2 * b + 1], A.kb[2 * (3 * a + b) + 1]);
-        A.gb[2 * (3 * a + b)] = fmaf(la, sg[2 * b], A.gb[2 * (3 * a + b)]);
-        A.gb[2 * (3 * a + b) + 1] = fmaf(la, sg[2 * b + 1], A.gb[2 * (3 * a + b) + 1]);
-      }
-      A.kp[2 * a] = fmaf(la, sx[0], A.kp[2 * a]);
-      A.kp[2 * a + 1] = fmaf(la, sx[1], A.kp[2 * a + 1]);
+      for (int b = 0; b < 3; ++b)
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          A.gb[2 * (3 * a + b) + i] = fmaf(la, sb[b][i], A.gb[2 * (3 * a + b) + i]);
+          A.ky[2 * (3 * a + b) + i] = fmaf(la, sb[b][2 + i], A.ky[2 * (3 * a + b) + i]);
+          A.kx[2 * (3 * a + b) + i] = fmaf(la, sb[b][4 + i], A.kx[2 * (3 * a + b) + i]);
+        }
     }
   }
   float cc[9];
@@ -306,9 +287,22 @@ k_gal_regular(const float4* __restrict__ c_hi, const float4* __restrict__ c_lo, 
       cc[3 * a + b] = ca.x * cb.x + ca.y * cb.y + ca.z * cb.z;
     }
   }
+  const float nn = nx.x * ny.x + nx.y * ny.y + nx.z * ny.z;
   float2 out[kGalVals];
-  gal_finish(A, k, nx.x * ny.x + nx.y * ny.y + nx.z * ny.z, cc, out);
-  gal_store(partL, partR, nt, blockIdx.y, s, out);
+  gal_finish<false>(A, k, nn, cc, out);
+  gal_store(partL, partR, nt, t - t0, s, out);
+  if (both) {
+    gal_finish<true>(A, k, nn, cc, out);
+#pragma unroll
+    for (int i = 0; i < kGalVals; ++i) s_st[i][lane][w] = out[i];
+  }
+  }
+  __syncthreads();
+  const int q = threadIdx.x % kGalT, e = threadIdx.x / kGalT;  // test triangle, s: 32 of them
+  if (s_ok[q] >> e & 1u) {
+#pragma unroll
+    for (int i = 0; i < kGalVals; ++i) gal_plane(partL, partR, nt, sb0 + e - t0, i)[tb + q] = s_st[i][e][q];
+  }
 }
 
 namespace {
@@ -324,7 +318,9 @@ __device__ __forceinline__ float3 f3sub(const double* a, const double* b) {
 }  // namespace
 
 // Pairs sharing a vertex or an edge (the near-pair list), then the identical pairs: one warp
-// per pair, the rule's points dealt over the lanes, a fixed shuffle tree, lane 0 writes.
+// per pair, the rule's points dealt over the lanes, a fixed shuffle tree, lane 0 writes. The rules
+// for (t, s) and (s, t) are the same points with the roles swapped (regions, signs and the
+// symmetric Gauss points trade places), so one warp forms both where both rows are in the round.
 __global__ void __launch_bounds__(256)
 k_gal_singular(const int2* __restrict__ near_pairs, int64_t n_near, const double* __restrict__ tri,
                const double* __restrict__ nrm64, const double* __restrict__ area, const int4* __restrict__ vid,
@@ -341,7 +337,7 @@ k_gal_singular(const int2* __restrict__ near_pairs, int64_t n_near, const double
   } else {
     t = s = (int)(w - n_near);
   }
-  if (t < t0 || t >= t1) return;
+  if (t < t0 || t >= t1 || (s >= t0 && s < t)) return;
   const double* Pt = tri + 9 * (size_t)t;
   const double* Ps = tri + 9 * (size_t)s;
   const double At = area[t], As = area[s];
@@ -456,19 +452,34 @@ k_gal_singular(const int2* __restrict__ near_pairs, int64_t n_near, const double
       gal_place(lam, ia, (ia + 1) % 3, 1.f - rt, rt * (1.f - thv), rt * thv);
       gal_place(mu, ja, (ja + 1) % 3, 1.f - rs, rs * (1.f - ths), rs * ths);
     }
-    const GalK v = gal_kernels(dx, dy, dz, k, gw * jac * jac_area, nx, ny);
-    gal_acc_point(A, lam, mu, v);
+    const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+    const float rinv = rsqrtf(r2), rho = k * (r2 * rinv);
+    float2 G, F;
+    gal_kernels(rinv, rho, gal_turns(rho), gw * jac * jac_area, G, F);
+    const float dny = fmaf(dx, ny.x, fmaf(dy, ny.y, dz * ny.z)), dnx = fmaf(dx, nx.x, fmaf(dy, nx.y, dz * nx.z));
+    const float v[6] = {G.x, G.y, F.x * dny, F.y * dny, F.x * dnx, F.y * dnx};
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+      for (int b = 0; b < 3; ++b) {
+        const float lm = lam[a] * mu[b];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          A.gb[2 * (3 * a + b) + i] = fmaf(lm, v[i], A.gb[2 * (3 * a + b) + i]);
+          A.ky[2 * (3 * a + b) + i] = fmaf(lm, v[2 + i], A.ky[2 * (3 * a + b) + i]);
+          A.kx[2 * (3 * a + b) + i] = fmaf(lm, v[4 + i], A.kx[2 * (3 * a + b) + i]);
+        }
+      }
   }
   // fixed-order reduction over the warp
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) {
 #pragma unroll
     for (int i = 0; i < 18; ++i) {
-      A.kb[i] += __shfl_xor_sync(0xffffffffu, A.kb[i], off);
       A.gb[i] += __shfl_xor_sync(0xffffffffu, A.gb[i], off);
+      A.ky[i] += __shfl_xor_sync(0xffffffffu, A.ky[i], off);
+      A.kx[i] += __shfl_xor_sync(0xffffffffu, A.kx[i], off);
     }
-#pragma unroll
-    for (int i = 0; i < 6; ++i) A.kp[i] += __shfl_xor_sync(0xffffffffu, A.kp[i], off);
   }
   if (lane != 0) return;
   float cc[9];
@@ -480,7 +491,8 @@ k_gal_singular(const int2* __restrict__ near_pairs, int64_t n_near, const double
     }
   }
   float2 out[kGalVals];
-  gal_finish(A, k, nx.x * ny.x + nx.y * ny.y + nx.z * ny.z, cc, out);
+  const float nn = nx.x * ny.x + nx.y * ny.y + nx.z * ny.z;
+  gal_finish<false>(A, k, nn, cc, out);
   if (kind == 3) {
     // mass terms: 1/2 M11 (A / 12 (1 + delta_ab)) and -(beta / 2) M10 (A / 3), beta = i / k
     const float m = (float)(At / 24.0);
@@ -489,6 +501,10 @@ k_gal_singular(const int2* __restrict__ near_pairs, int64_t n_near, const double
     for (int a = 0; a < 3; ++a) out[9 + a].y -= (float)(At / 6.0) / k;
   }
   gal_store(partL, partR, nt, t - t0, s, out);
+  if (s > t && s < t1) {
+    gal_finish<true>(A, k, nn, cc, out);
+    gal_store(partL, partR, nt, s - t0, t, out);
+  }
 }
 
 // First stage of the L gather, one block row per test triangle tau of the round: for every
@@ -501,14 +517,14 @@ k_gal_rowsum_L(const float2* __restrict__ partL, int nt, const int* __restrict__
   const int tr = blockIdx.y;
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= nv) return;
-  const float2* row = partL + (size_t)tr * nt * 9;
+  const float2* row = partL + (size_t)tr * 9 * nt;
   float2 acc[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
   for (int v = adj_ptr[j]; v < adj_ptr[j + 1]; ++v) {
     const int2 sb = adj[v];
-    const float2* blk = row + (size_t)sb.x * 9 + sb.y;
+    const float2* blk = row + (size_t)sb.y * nt + sb.x;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      const float2 x = blk[3 * a];
+      const float2 x = blk[(size_t)3 * a * nt];
       acc[a].x += x.x;
       acc[a].y += x.y;
     }
@@ -661,8 +677,8 @@ nat_bem_status galerkin_assemble_operators(nat_bem_op* op, cudaStream_t s) {
   for (int t0 = 0; t0 < nt && st == NAT_BEM_OK; t0 += chunk) {
     const int t1 = std::min(nt, t0 + chunk);
     const bool last = t1 == nt;
-    NB_LAUNCH("gal_regular", s, k_gal_regular<<<dim3((unsigned)((nt + 255) / 256), (unsigned)(t1 - t0)), 256, 0, s>>>(
-        g.c_hi, g.c_lo, g.nrm, g.qp, g.vid, G.curl, nt, t0, k, partL, partR));
+    NB_LAUNCH("gal_regular", s, k_gal_regular<<<dim3((unsigned)((nt + 31) / 32), (unsigned)((t1 - t0 + kGalT - 1) / kGalT)), kGalT * 32, 0, s>>>(
+        g.c_hi, g.c_lo, g.nrm, g.qp, g.vid, G.curl, nt, t0, t1, k, partL, partR));
     const int64_t warps = g.n_near + nt;
     NB_LAUNCH("gal_singular", s, k_gal_singular<<<(unsigned)((warps * 32 + 255) / 256), 256, 0, s>>>(
         g.near_pairs, g.n_near, g.tri, g.nrm64, g.area, g.vid, G.curl, nt, t0, t1, k, partL, partR));

@@ -146,3 +146,23 @@ def test_galerkin_rejects_bad_input(nb):
         nb.Operator.assemble_galerkin(Vx, F, 1.0)
     with pytest.raises(nb.NatBemError):
         nb.Operator.assemble_galerkin(V, F, -1.0)
+
+
+def test_two_rounds_of_test_triangles_sampled_rows(nb):
+    """More triangles than one round of pair blocks holds: a pair in one round is formed once for
+    both directions, a pair across rounds once per direction. Rows of vertices in the first round,
+    in the second and on the boundary."""
+    from oracle import galerkin as G
+    Vs, F = S.ring_sphere(6600)
+    V = S.perturbed_ellipsoid(Vs, 5)
+    k = 2.5
+    nt, nv, ldv = len(F), len(V), (len(V) + 31) // 32 * 32
+    first = int(4e9 / (nt * 96 + 3 * ldv * 8))  # triangles of the first round
+    assert 512 < first < nt - 300
+    rows = np.unique(np.concatenate([F[0], F[first - 1], F[first], F[nt - 1]]))[[0, 2, 5, -1]]
+    Lr, Rr = G.assemble_rows(V, F, k, rows)
+    with nb.Operator.assemble_galerkin(V, F, k) as op:
+        for i, r in enumerate(rows):
+            L, R = op.rows(0, int(r), 1)[0], op.rows(1, int(r), 1)[0]
+            assert np.linalg.norm(L[:nv] - Lr[i]) / np.linalg.norm(Lr[i]) < 1e-5
+            assert np.linalg.norm(R[:nt] - Rr[i]) / np.linalg.norm(Rr[i]) < 1e-5
