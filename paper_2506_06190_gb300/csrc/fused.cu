@@ -66,7 +66,7 @@ int64_t op_bytes(int64_t N, bool bf16) {
 }
 
 // One bucket: assemble every mesh into its slice, pad, solve all in lockstep, evaluate fields.
-nat_bem_status run_bucket(nat_bem_job* jobs, const Bucket& bk, const nat_bem_opts& o, cudaStream_t s,
+nat_bem_status run_bucket(nat_bem_job* jobs, const Bucket& bk, const nat_bem_opts& o, int share, cudaStream_t s,
                           std::string& first_error) {
   const int B = (int)bk.jobs.size();
   const int64_t N = bk.N, ld = round_up(N, 32);
@@ -76,6 +76,8 @@ nat_bem_status run_bucket(nat_bem_job* jobs, const Bucket& bk, const nat_bem_opt
   float2 *L = nullptr, *R = nullptr, *G = nullptr, *P = nullptr;
   uint32_t* Lb = nullptr;
   float* RS = nullptr;
+  int* rows = nullptr;
+  std::vector<int> hrows(B, 0);
   std::vector<nat_bem_op*> ops(B, nullptr);
   nat_bem_op* batch = nullptr;
   cudaEvent_t t0 = nullptr, t1 = nullptr;
@@ -88,6 +90,7 @@ nat_bem_status run_bucket(nat_bem_job* jobs, const Bucket& bk, const nat_bem_opt
     dev_free(RS, s);
     dev_free(G, s);
     dev_free(P, s);
+    dev_free(rows, s);
     if (t0) cudaEventDestroy(t0);
     if (t1) cudaEventDestroy(t1);
   };
@@ -101,6 +104,7 @@ nat_bem_status run_bucket(nat_bem_job* jobs, const Bucket& bk, const nat_bem_opt
   if ((st = dev_alloc_n(&L, slice * B, s)) != NAT_BEM_OK || (st = dev_alloc_n(&R, slice * B, s)) != NAT_BEM_OK ||
       (bf16 && (st = dev_alloc_n(&Lb, slice * B, s)) != NAT_BEM_OK) ||
       (fp16 && (st = dev_alloc_n(&RS, (size_t)N * B, s)) != NAT_BEM_OK) ||
+      (st = dev_alloc_n(&rows, (size_t)B, s)) != NAT_BEM_OK ||
       (st = dev_alloc_n(&G, (size_t)N * B, s)) != NAT_BEM_OK || (st = dev_alloc_n(&P, (size_t)N * B, s)) != NAT_BEM_OK)
     return fail_all(st);
   if (cudaEventCreate(&t0) != cudaSuccess || cudaEventCreate(&t1) != cudaSuccess) {
@@ -150,6 +154,7 @@ nat_bem_status run_bucket(nat_bem_job* jobs, const Bucket& bk, const nat_bem_opt
     } else {
       ok[b] = 1;
     }
+    hrows[b] = std::max(n_b, 1);
     if (n_b < N) {
       const int64_t tot = (int64_t)(N - n_b) * ld;
       NB_LAUNCH("pad_rows", s, k_pad_rows<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(
@@ -189,6 +194,12 @@ nat_bem_status run_bucket(nat_bem_job* jobs, const Bucket& bk, const nat_bem_opt
   batch->copy_fp16 = fp16;
   batch->row_scale = RS;
   batch->bstride = (int64_t)slice;
+  if (cudaMemcpyAsync(rows, hrows.data(), B * sizeof(int), cudaMemcpyHostToDevice, s) != cudaSuccess) {
+    set_error("run_batch_fused: copy of the row counts failed");
+    return fail_all(NAT_BEM_ECUDA);
+  }
+  batch->batch_n = rows;
+  batch->share = share;
   std::vector<nat_bem_solve_info> per;
   std::vector<int> conv;
   nat_bem_solve_info info{};
@@ -303,7 +314,7 @@ extern "C" nat_bem_status nat_bem_run_batch_fused(nat_bem_job* jobs, int32_t njo
         if (it >= items) break;
         std::string err;
         if (it < (int)buckets.size()) {
-          run_bucket(jobs, buckets[it], o, s, err);
+          run_bucket(jobs, buckets[it], o, nw, s, err);
         } else {
           nat_bem_job& j = jobs[single[it - buckets.size()]];
           nat_bem_op* op = nullptr;

@@ -23,6 +23,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdlib>
+#include <cstring>
 #include <map>
 #include <tuple>
 #include <mutex>
@@ -73,12 +74,22 @@ struct Workspace {
   bool loops_off = false;
   unsigned long long* loop_launches = nullptr;  // kernels the loop bodies ran (device counter)
   int* loop_bodies = nullptr;                    // bodies the current loop ran (reset per run)
-  unsigned long long* host_loop = nullptr;      // pinned mirror, read at host sync points
+  bool loop_ran = false;                         // a loop ran since the last host sync point
   void* tc_scratch = nullptr;                              // packed B + split-K partials
   size_t tc_bytes = 0;
   int* tc_err = nullptr;                                   // bounded-wait failures
   unsigned* cnt = nullptr;
-  int* host_scal = nullptr;  // pinned mirror of scal[0..1]
+  char* arena = nullptr;     // every device array above, one allocation
+  // What the host reads and what a solve starts from zero, side by side: one copy to the pinned
+  // mirror per host sync point and one memset per solve
+  //   res_true, loop_launches, iters, done | outer_done, tc_err | gbar
+  //   read ................................................... |
+  //                                          zeroed .............................
+  bool pending = false;      // copies to the mirror enqueued, not yet waited for
+  size_t status_read = 0, status_zero_at = 0, status_zero = 0;
+  char* status = nullptr;
+  char* host = nullptr;      // pinned mirror of the status, then of scal[0..1]
+  int* host_scal = nullptr;
 };
 
 struct GArgs {
@@ -1884,11 +1895,24 @@ static const void* run_kernel(int fmt, bool f32) {
   }
 }
 
-// Shape of k_gmres_run for an operator of `n` rows (stages = 0: it does not fit) and its grid:
-// one block per SM, at least eight rows a block.
-static RunArgs run_fit(int n, int ld, int blocks, int fmt, bool f32, int cols, int* grid) {
-  *grid = std::max(1, std::min(blocks, (n + 7) / 8));
-  return run_shape(n, ld, *grid, fmt, f32, cols);
+// Shape of k_gmres_run for `systems` systems of up to n rows (stages = 0: one does not fit): how many
+// go into one launch and the blocks of each, one block per SM in all. One system gets as many blocks
+// as leave it eight rows each. Several, or several launches in flight (`share`), divide the SMs as long
+// as a block keeps about 64 rows: one's matvec streams while another waits in Gram-Schmidt.
+static RunArgs run_fit(int n, int ld, int blocks, int systems, int share, int fmt, bool f32, int cols, int* at_once) {
+  RunArgs r{};
+  const int most = (n + 63) / 64;  // blocks of a system that shares the SMs
+  for (int k = std::max(1, std::min(systems, blocks / most)); k >= 1; --k)
+    for (int f = share; f >= 1; f = f > 1 ? 1 : 0) {
+      int each = blocks / k;
+      if (f > 1) each = std::min(each, std::max(blocks / (k * f), most));
+      each = std::max(1, std::min(each, (n + 7) / 8));
+      r = run_shape(n, ld, each, fmt, f32, cols);
+      r.blocks = each;
+      *at_once = k;
+      if (r.stages > 0) return r;
+    }
+  return r;
 }
 
 // Whether every form of the kernel is launchable on the current device.
@@ -1950,21 +1974,58 @@ int64_t workspace_bytes(int64_t n, int nrhs, const nat_bem_opts& o) {
   return b;
 }
 
+// Pinned host memory for the workspaces' mirrors: slots of one page-locked block per process, so
+// that short-lived ops (a batch builds one per mesh) don't allocate and free page-locked memory,
+// which waits for the whole device. A mirror larger than a slot, or with every slot taken, is
+// allocated by itself.
+namespace {
+constexpr size_t kPinSlot = 4096;
+constexpr int kPinSlots = 64;
+std::mutex g_pin_mu;
+char* g_pin_base = nullptr;
+bool g_pin_used[kPinSlots] = {};
+
+char* pin_take(size_t bytes) {
+  if (bytes <= kPinSlot) {
+    std::lock_guard<std::mutex> lk(g_pin_mu);
+    if (!g_pin_base && cudaHostAlloc(reinterpret_cast<void**>(&g_pin_base), kPinSlot * kPinSlots,
+                                     cudaHostAllocPortable) != cudaSuccess) {
+      cudaGetLastError();
+      g_pin_base = nullptr;
+    }
+    for (int i = 0; g_pin_base && i < kPinSlots; ++i)
+      if (!g_pin_used[i]) {
+        g_pin_used[i] = true;
+        return g_pin_base + i * kPinSlot;
+      }
+  }
+  void* p = nullptr;
+  if (cudaHostAlloc(&p, bytes, cudaHostAllocPortable) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  return static_cast<char*>(p);
+}
+void pin_give(char* p) {
+  if (!p) return;
+  {
+    std::lock_guard<std::mutex> lk(g_pin_mu);
+    if (g_pin_base && p >= g_pin_base && p < g_pin_base + kPinSlot * kPinSlots) {
+      g_pin_used[(p - g_pin_base) / kPinSlot] = false;
+      return;
+    }
+  }
+  cudaFreeHost(p);
+}
+}  // namespace
+
 void workspace_free(Workspace* ws, cudaStream_t s) {
   if (!ws) return;
-  void* ptrs[] = {ws->b, ws->V, ws->w, ws->x, ws->H, ws->hcol, ws->htmp, ws->sn, ws->gv, ws->y,
-                  ws->part, ws->cs, ws->partn, ws->bnorm, ws->res, ws->hnorm, ws->res_true,
-                  ws->xf, ws->gin, ws->pout, ws->done, ws->iters, ws->scal, ws->cnt,
-                  ws->b0, ws->xacc, ws->b0norm, ws->outer_done, ws->tc_scratch, ws->tc_err, ws->gbar,
-                  ws->pblk, ws->hred, ws->pbu, ws->wf};
-  for (void* p : ptrs)
-    if (p) dev_free(p, s);
-  if (ws->host_scal) cudaFreeHost(ws->host_scal);
+  if (ws->pending) cudaDeviceSynchronize();  // a failed call left copies to the mirror in flight
+  dev_free(ws->arena, s);
+  pin_give(ws->host);
   for (auto& kv : ws->graphs) cudaGraphExecDestroy(kv.second.first);
   for (auto& kv : ws->loops) cudaGraphExecDestroy(kv.second);
-  if (ws->loop_launches) dev_free(ws->loop_launches, s);
-  if (ws->loop_bodies) dev_free(ws->loop_bodies, s);
-  if (ws->host_loop) cudaFreeHost(ws->host_loop);
   delete ws;
 }
 
@@ -1985,40 +2046,41 @@ static nat_bem_status workspace_ensure(nat_bem_op* op, int nrhs, cudaStream_t s)
   ws->m = m;
   ws->nchunk = (int)((n + kUpdRows - 1) / kUpdRows);
   const size_t nr = (size_t)nrhs, mm = (size_t)m;
-  NB_TRY(dev_alloc_n(&ws->b, n * nr, s));
-  NB_TRY(dev_alloc_n(&ws->w, n * nr, s));
-  NB_TRY(dev_alloc_n(&ws->x, n * nr, s));
-  NB_TRY(dev_alloc_n(&ws->V, n * nr * (mm + 1), s));
-  NB_TRY(dev_alloc_n(&ws->H, nr * mm * (mm + 1), s));
-  NB_TRY(dev_alloc_n(&ws->hcol, nr * (mm + 1), s));
-  NB_TRY(dev_alloc_n(&ws->htmp, nr * (mm + 1), s));
-  NB_TRY(dev_alloc_n(&ws->sn, nr * mm, s));
-  NB_TRY(dev_alloc_n(&ws->gv, nr * (mm + 1), s));
-  NB_TRY(dev_alloc_n(&ws->y, nr * mm, s));
-  NB_TRY(dev_alloc_n(&ws->part, std::max<size_t>((size_t)ws->nchunk, kDotChunks) * nr * (mm + 1), s));
-  NB_TRY(dev_alloc_n(&ws->cs, nr * mm, s));
-  NB_TRY(dev_alloc_n(&ws->partn, (size_t)ws->nchunk * nr, s));
-  NB_TRY(dev_alloc_n(&ws->bnorm, nr, s));
-  NB_TRY(dev_alloc_n(&ws->res, nr, s));
-  NB_TRY(dev_alloc_n(&ws->hnorm, nr, s));
-  NB_TRY(dev_alloc_n(&ws->res_true, nr, s));
-  NB_TRY(dev_alloc_n(&ws->xf, ld * nr, s));
-  NB_TRY(dev_alloc_n(&ws->gin, std::max<int64_t>(ld, op->ldr) * nr, s));
-  NB_TRY(dev_alloc_n(&ws->pout, n * nr, s));
-  NB_TRY(dev_alloc_n(&ws->done, nr, s));
-  NB_TRY(dev_alloc_n(&ws->iters, nr, s));
-  NB_TRY(dev_alloc_n(&ws->scal, 4, s));
-  NB_TRY(dev_alloc_n(&ws->cnt, nr * kCounters, s));
-  NB_TRY(dev_alloc_n(&ws->b0, n * nr, s));
-  NB_TRY(dev_alloc_n(&ws->xacc, n * nr, s));
-  NB_TRY(dev_alloc_n(&ws->b0norm, nr, s));
-  NB_TRY(dev_alloc_n(&ws->outer_done, nr, s));
-  NB_TRY(dev_alloc_n(&ws->tc_err, 1, s));
-  NB_TRY(dev_alloc_n(&ws->gbar, 2, s));
-  NB_TRY(dev_alloc_n(&ws->loop_launches, 1, s));
-  NB_TRY(dev_alloc_n(&ws->loop_bodies, 1, s));
-  NB_TRY_CUDA(cudaMemsetAsync(ws->loop_launches, 0, sizeof(unsigned long long), s));
-  NB_TRY_CUDA(cudaMemsetAsync(ws->gbar, 0, 2 * sizeof(unsigned), s));
+  // every device array, laid out one after another in a single allocation
+  std::vector<std::pair<void**, size_t>> arrays;
+  size_t total = 0;
+  auto take = [&](auto** p, size_t count) {
+    arrays.emplace_back(reinterpret_cast<void**>(p), total);
+    total += (std::max<size_t>(count, 1) * sizeof(**p) + 255) / 256 * 256;
+  };
+  take(&ws->b, n * nr);
+  take(&ws->w, n * nr);
+  take(&ws->x, n * nr);
+  take(&ws->V, n * nr * (mm + 1));
+  take(&ws->H, nr * mm * (mm + 1));
+  take(&ws->hcol, nr * (mm + 1));
+  take(&ws->htmp, nr * (mm + 1));
+  take(&ws->sn, nr * mm);
+  take(&ws->gv, nr * (mm + 1));
+  take(&ws->y, nr * mm);
+  take(&ws->part, std::max<size_t>((size_t)ws->nchunk, kDotChunks) * nr * (mm + 1));
+  take(&ws->cs, nr * mm);
+  take(&ws->partn, (size_t)ws->nchunk * nr);
+  take(&ws->bnorm, nr);
+  take(&ws->res, nr);
+  take(&ws->hnorm, nr);
+  take(&ws->xf, ld * nr);
+  take(&ws->gin, std::max<int64_t>(ld, op->ldr) * nr);
+  take(&ws->pout, n * nr);
+  take(&ws->scal, 4);
+  take(&ws->cnt, nr * kCounters);
+  take(&ws->b0, n * nr);
+  take(&ws->xacc, n * nr);
+  take(&ws->b0norm, nr);
+  take(&ws->loop_bodies, 1);
+  const size_t st_iters = 8 * nr + 8, st_zero = st_iters + 8 * nr, st_read = st_zero + 4 * nr + 4;
+  const size_t st_all = (st_read + 7) / 8 * 8 + 8 * nr;
+  take(&ws->status, st_all);
   {
     // the fused Arnoldi kernel runs one block per SM when every block fits at once and the
     // rows per block and the RHS count fit its shared-memory staging
@@ -2056,8 +2118,8 @@ static nat_bem_status workspace_ensure(nat_bem_op* op, int nrhs, cudaStream_t s)
     const bool fits = sms >= 2 && n <= (int64_t)(sms - 1) * kArnMaxRows && nrhs <= kArnMaxRhs;
     ws->coop_blocks = (coop && per_sm >= 1 && fits && !std::getenv("NATBEM_NO_FUSED_KRYLOV")) ? sms : 0;
     if (ws->coop_blocks > 0) {
-      NB_TRY(dev_alloc_n(&ws->pblk, nr * (mm + 2) * (size_t)ws->coop_blocks, s));
-      NB_TRY(dev_alloc_n(&ws->hred, nr * (mm + 2), s));
+      take(&ws->pblk, nr * (mm + 2) * (size_t)ws->coop_blocks);
+      take(&ws->hred, nr * (mm + 2));
       if (nrhs > kArnUnitsMinRhs) {  // the multi-RHS kernel: partials for the largest unit count
         // its own grid: up to kArnUnitsPerSm blocks per SM (more loads in flight for the
         // streaming dots and row updates; one block per SM kept about a third of the HBM rate)
@@ -2070,26 +2132,49 @@ static nat_bem_status workspace_ensure(nat_bem_op* op, int nrhs, cudaStream_t s)
           const int u = arnoldi_unit((int)n, q, ws->units_blocks);
           most = std::max(most, (size_t)q * (size_t)((n + u - 1) / u));
         }
-        NB_TRY(dev_alloc_n(&ws->pbu, most * (mm + 2), s));
+        take(&ws->pbu, most * (mm + 2));
       }
-      NB_TRY(dev_alloc_n(&ws->wf, (size_t)n * nr, s));  // FP32 w of inner solves on the FP32 basis
-      ws->run_ok = nrhs == 1 && op->bstride == 0 && !std::getenv("NATBEM_NO_RUN_KERNEL") && run_usable();
+      take(&ws->wf, (size_t)n * nr);  // FP32 w of inner solves on the FP32 basis
+      ws->run_ok = (nrhs == 1 || op->bstride > 0) && !std::getenv("NATBEM_NO_RUN_KERNEL") && run_usable();
     }
   }
-  NB_TRY_CUDA(cudaMemsetAsync(ws->tc_err, 0, sizeof(int), s));
+  char* tc = nullptr;
   if (nrhs > 1) {
     int dev = 0, sms = 148;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     ws->tc_bytes = tc_workspace_bytes(n, std::max<int64_t>(ld, op->ldr), nrhs, sms);  // L and R products
-    NB_TRY(dev_alloc(&ws->tc_scratch, ws->tc_bytes, s));
+    take(&tc, ws->tc_bytes);
   }
+  ws->host = pin_take((st_read + 15) / 16 * 16 + 16);
+  nat_bem_status got = NAT_BEM_OK;
+  if (!ws->host) {
+    set_error("page-locked host allocation failed");
+    got = NAT_BEM_ENOMEM;
+  }
+  if (got == NAT_BEM_OK) got = dev_alloc_n(&ws->arena, total, s);
+  if (got != NAT_BEM_OK) {  // no half-built workspace for a later call to find
+    workspace_free(ws, s);
+    op->ws = nullptr;
+    return got;
+  }
+  for (auto& p : arrays) *p.first = ws->arena + p.second;
+  ws->tc_scratch = tc;
+  ws->res_true = reinterpret_cast<double*>(ws->status);
+  ws->loop_launches = reinterpret_cast<unsigned long long*>(ws->status + 8 * nr);
+  ws->iters = reinterpret_cast<int*>(ws->status + st_iters);
+  ws->done = ws->iters + nr;
+  ws->outer_done = ws->done + nr;
+  ws->tc_err = ws->outer_done + nr;
+  ws->gbar = reinterpret_cast<unsigned*>(ws->status + (st_read + 7) / 8 * 8);
+  ws->status_read = st_read;
+  ws->status_zero_at = st_zero;
+  ws->status_zero = st_all - st_zero;
+  NB_TRY_CUDA(cudaMemsetAsync(ws->status, 0, st_all, s));
   NB_TRY_CUDA(cudaMemsetAsync(ws->cnt, 0, nr * kCounters * sizeof(unsigned), s));
   NB_TRY_CUDA(cudaMemsetAsync(ws->scal, 0, 4 * sizeof(int), s));
   NB_TRY_CUDA(cudaMemsetAsync(ws->xf, 0, ld * nr * sizeof(float2), s));
-  NB_TRY_CUDA(cudaMallocHost(&ws->host_scal, 4 * sizeof(int)));
-  NB_TRY_CUDA(cudaMallocHost(&ws->host_loop, sizeof(unsigned long long)));
-  *ws->host_loop = 0;
+  ws->host_scal = reinterpret_cast<int*>(ws->host + (st_read + 15) / 16 * 16);
   return NAT_BEM_OK;
 }
 
@@ -2441,15 +2526,26 @@ __global__ void k_loop_cond(cudaGraphConditionalHandle h, const int* __restrict_
   }
 }
 
-// Kernels the device-side loops ran, for the launch counter: loop_copy enqueues the read of the
-// device counter (and its reset) before a host sync point, loop_count adds it after the sync.
-static void loop_copy(Workspace* ws, cudaStream_t s) {
-  cudaMemcpyAsync(ws->host_loop, ws->loop_launches, sizeof(unsigned long long), cudaMemcpyDeviceToHost, s);
-  cudaMemsetAsync(ws->loop_launches, 0, sizeof(unsigned long long), s);
+// One host sync point: the status block to its pinned mirror, and the kernels the device-side loops
+// ran to the launch counter.
+static nat_bem_status status_sync(Workspace* ws, cudaStream_t s) {
+  ws->pending = true;
+  NB_TRY_CUDA(cudaMemcpyAsync(ws->host, ws->status, ws->status_read, cudaMemcpyDeviceToHost, s));
+  if (ws->loop_ran) NB_TRY_CUDA(cudaMemsetAsync(ws->loop_launches, 0, sizeof(unsigned long long), s));
+  NB_TRY_CUDA(cudaStreamSynchronize(s));
+  ws->pending = false;
+  if (ws->loop_ran) {
+    unsigned long long n;
+    std::memcpy(&n, ws->host + ((char*)ws->loop_launches - ws->status), sizeof(n));
+    add_launches((int64_t)n);
+    ws->loop_ran = false;
+  }
+  return NAT_BEM_OK;
 }
-static void loop_count(Workspace* ws) {
-  add_launches((int64_t)*ws->host_loop);
-  *ws->host_loop = 0;
+// `count` values of a device array of the status block, from the mirror.
+template <class T>
+static void status_get(const Workspace* ws, const T* dev, T* out, int count) {
+  std::memcpy(out, ws->host + (reinterpret_cast<const char*>(dev) - ws->status), count * sizeof(T));
 }
 
 static nat_bem_status gmres_run(nat_bem_op* op, Workspace* ws, const GArgs& a, int engine,
@@ -2461,24 +2557,33 @@ static nat_bem_status gmres_run(nat_bem_op* op, Workspace* ws, const GArgs& a, i
   // times). Measured with one solve in flight, two-launch form -> this, a whole solve: 1280 rows
   // FP32 1037 -> 478 us, 3956 783 -> 466, 5174 1888 -> 1401, 10240 5878 -> 4299; 10240 mixed BF16
   // 4283 -> 3643. Above that the matvec streams for 10x the time of the rest of an iteration.
-  if (ws->run_ok && nrhs == 1 && op->bstride == 0 && !tracing_enabled()) {
+  if (ws->run_ok && (engine == kEngineGemv || engine == kEngineGemvCopy) && !tracing_enabled()) {
     const int fmt = engine == kEngineGemv ? 0 : (op->copy_fp16 ? 2 : 1);
-    int grid = 0;
-    RunArgs r = run_fit(n, (int)ws->ld, ws->coop_blocks, fmt, a.Vf != nullptr, a.maxit + 1, &grid);
-    if (r.stages > 0) {
-      r.A = fmt == 0 ? (const void*)op->L : (const void*)op->Lb;
-      r.rs = fmt == 2 ? op->row_scale : nullptr;
-      r.pb = ws->pblk;
-      r.hr = ws->hred;
-      r.bar = ws->gbar;
-      r.err = ws->tc_err;
-      r.pout = pout;
-      r.accumulate = accumulate;
-      GArgs ac = a;
-      void* args[] = {&ac, &r};
-      NB_LAUNCH("gmres_run", s, NB_TRY_CUDA(cudaLaunchCooperativeKernel(run_kernel(fmt, a.Vf != nullptr), dim3(grid),
-                                                                       dim3(kRunThreads), args, (size_t)kRunSmem, s)));
-      NB_CHECK_LAUNCH();
+    int at_once = 1;
+    const RunArgs shape = run_fit(n, (int)ws->ld, ws->coop_blocks, nrhs, std::max(1, op->share), fmt, a.Vf != nullptr,
+                                  a.maxit + 1, &at_once);
+    if (shape.stages > 0) {
+      for (int s0 = 0; s0 < nrhs; s0 += at_once) {
+        RunArgs r = shape;
+        r.s0 = s0;
+        r.ns = op->batch_n;
+        r.astride = op->bstride;
+        r.sstride = op->bstride > 0 ? n : 0;
+        r.A = fmt == 0 ? (const void*)op->L : (const void*)op->Lb;
+        r.rs = fmt == 2 ? op->row_scale : nullptr;
+        r.pb = ws->pblk;
+        r.hr = ws->hred;
+        r.bar = ws->gbar;
+        r.err = ws->tc_err;
+        r.pout = pout;
+        r.accumulate = accumulate;
+        GArgs ac = a;
+        void* args[] = {&ac, &r};
+        const int grid = std::min(at_once, nrhs - s0) * r.blocks;
+        NB_LAUNCH("gmres_run", s, NB_TRY_CUDA(cudaLaunchCooperativeKernel(run_kernel(fmt, a.Vf != nullptr), dim3(grid),
+                                                                         dim3(kRunThreads), args, (size_t)kRunSmem, s)));
+        NB_CHECK_LAUNCH();
+      }
       return NAT_BEM_OK;
     }
   }
@@ -2580,6 +2685,7 @@ static nat_bem_status gmres_run(nat_bem_op* op, Workspace* ws, const GArgs& a, i
     if (f != ws->loops.end()) {
       NB_TRY_CUDA(cudaMemsetAsync(ws->loop_bodies, 0, sizeof(int), s));
       NB_TRY_CUDA(cudaGraphLaunch(f->second, s));
+      ws->loop_ran = true;
       const dim3 vg((n + kChunk - 1) / kChunk, nrhs);
       NB_LAUNCH("gmres_lsq", s, k_lsq<<<nrhs, 256, 0, s>>>(a));
       NB_LAUNCH("gmres_xupdate", s, k_xupdate<<<vg, kChunk, 0, s>>>(a, pout, accumulate));
@@ -2621,8 +2727,10 @@ static nat_bem_status gmres_run(nat_bem_op* op, Workspace* ws, const GArgs& a, i
     if (done_direct) NB_TRY(launch_chunk(it, c));
     NB_CHECK_LAUNCH();
     it += c;
+    ws->pending = true;
     NB_TRY_CUDA(cudaMemcpyAsync(ws->host_scal, ws->scal, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
     NB_TRY_CUDA(cudaStreamSynchronize(s));
+    ws->pending = false;
     if (ws->host_scal[1]) break;
     chunk = 8;
   }
@@ -2714,8 +2822,8 @@ nat_bem_status solve_impl(nat_bem_op* op, const float2* d_neumann, int nrhs, flo
   if (nrhs >= kX6MinRhs && op->bstride == 0 && x6_enabled()) NB_TRY(ensure_split(op, s));
   Workspace* ws = op->ws;
   const nat_bem_opts& o = op->opts;
-  NB_TRY_CUDA(cudaMemsetAsync(ws->gbar, 0, 2 * sizeof(unsigned), s));
-  NB_TRY_CUDA(cudaMemsetAsync(ws->tc_err, 0, sizeof(int), s));  // this solve's bounded-wait flags
+  // this solve's bounded-wait flags, barriers and refinement flags
+  NB_TRY_CUDA(cudaMemsetAsync(ws->status + ws->status_zero_at, 0, ws->status_zero, s));
   const int n = (int)op->n;
   const dim3 vec_grid((n + kChunk - 1) / kChunk, nrhs);
   // b = R g
@@ -2763,13 +2871,11 @@ nat_bem_status solve_impl(nat_bem_op* op, const float2* d_neumann, int nrhs, flo
     NB_TRY(matvec(op, ws, 0, accurate, ws->w, nullptr, nullptr, "gemv_resid", s));
     NB_LAUNCH("gmres_resid", s, k_resid<<<vec_grid, kChunk, 0, s>>>(a));
     NB_CHECK_LAUNCH();
-    NB_TRY_CUDA(cudaMemcpyAsync(iters.data(), ws->iters, nrhs * sizeof(int), cudaMemcpyDeviceToHost, s));
-    NB_TRY_CUDA(cudaMemcpyAsync(done.data(), ws->done, nrhs * sizeof(int), cudaMemcpyDeviceToHost, s));
-    NB_TRY_CUDA(cudaMemcpyAsync(rt.data(), ws->res_true, nrhs * sizeof(double), cudaMemcpyDeviceToHost, s));
-    NB_TRY_CUDA(cudaMemcpyAsync(&tc_err, ws->tc_err, sizeof(int), cudaMemcpyDeviceToHost, s));
-    loop_copy(ws, s);
-    NB_TRY_CUDA(cudaStreamSynchronize(s));  // the solve's one host sync
-    loop_count(ws);
+    NB_TRY(status_sync(ws, s));  // the solve's one host sync
+    status_get(ws, ws->iters, iters.data(), nrhs);
+    status_get(ws, ws->done, done.data(), nrhs);
+    status_get(ws, ws->res_true, rt.data(), nrhs);
+    status_get(ws, ws->tc_err, &tc_err, 1);
     for (int q = 0; q < nrhs; ++q) {
       total[q] = iters[q];
       conv[q] = done[q];
@@ -2781,7 +2887,6 @@ nat_bem_status solve_impl(nat_bem_op* op, const float2* d_neumann, int nrhs, flo
     // each sweep solves the correction equation L d = b with GMRES from d = 0, x += d.
     NB_TRY_CUDA(cudaMemcpyAsync(ws->b0, ws->b, (size_t)n * nrhs * sizeof(double2), cudaMemcpyDeviceToDevice, s));
     NB_TRY_CUDA(cudaMemsetAsync(ws->xacc, 0, (size_t)n * nrhs * sizeof(double2), s));
-    NB_TRY_CUDA(cudaMemsetAsync(ws->outer_done, 0, nrhs * sizeof(int), s));
     GArgs a = make_args(op, ws, op->L);
     a.x = ws->xacc;
     a.skip = ws->outer_done;
@@ -2801,14 +2906,12 @@ nat_bem_status solve_impl(nat_bem_op* op, const float2* d_neumann, int nrhs, flo
       NB_TRY(matvec(op, ws, 0, accurate, ws->w, nullptr, nullptr, "gemv_resid", s));
       NB_LAUNCH("ir_residual", s, k_ir_residual<<<vec_grid, kChunk, 0, s>>>(a, ws->b0, ws->outer_done, o.tol));
       NB_CHECK_LAUNCH();
-      NB_TRY_CUDA(cudaMemcpyAsync(iters.data(), ws->iters, nrhs * sizeof(int), cudaMemcpyDeviceToHost, s));
-      NB_TRY_CUDA(cudaMemcpyAsync(od.data(), ws->outer_done, nrhs * sizeof(int), cudaMemcpyDeviceToHost, s));
-      NB_TRY_CUDA(cudaMemcpyAsync(inner_done.data(), ws->done, nrhs * sizeof(int), cudaMemcpyDeviceToHost, s));
-      NB_TRY_CUDA(cudaMemcpyAsync(rt.data(), ws->res_true, nrhs * sizeof(double), cudaMemcpyDeviceToHost, s));
-      NB_TRY_CUDA(cudaMemcpyAsync(&tc_err, ws->tc_err, sizeof(int), cudaMemcpyDeviceToHost, s));
-      loop_copy(ws, s);
-      NB_TRY_CUDA(cudaStreamSynchronize(s));  // one host sync per sweep
-      loop_count(ws);
+      NB_TRY(status_sync(ws, s));  // one host sync per sweep
+      status_get(ws, ws->iters, iters.data(), nrhs);
+      status_get(ws, ws->outer_done, od.data(), nrhs);
+      status_get(ws, ws->done, inner_done.data(), nrhs);
+      status_get(ws, ws->res_true, rt.data(), nrhs);
+      status_get(ws, ws->tc_err, &tc_err, 1);
       if (tc_err) {
         set_error("GMRES: a bounded wait gave up (code " + std::to_string(tc_err) + ")");
         return NAT_BEM_ECUDA;

@@ -1,4 +1,6 @@
-// A whole GMRES run for one right-hand side in one cooperative launch (included by gmres.cu).
+// A whole GMRES run for one right-hand side, or for several systems of one each (a batch of
+// operators, each system on blocks of its own and as long as it needs), in one cooperative launch
+// (included by gmres.cu).
 //
 // The two-launch iteration (matvec, k_arnoldi) is bound by latency below a few thousand rows:
 // every iteration pays two kernel starts and drains, reloads the Krylov basis, and leaves HBM
@@ -46,6 +48,11 @@ template <int kFmt>
 constexpr int kRunSlots = kFmt == 0 ? 10 : 6;
 
 struct RunArgs {
+  int blocks;        // blocks per system; block b works on system s0 + b / blocks
+  int s0;            // first system of the launch
+  const int* ns;     // rows of each system, or null: n
+  int64_t astride;   // operators of a batch: elements of A from one to the next (0: one system)
+  int64_t sstride;   // row scales likewise
   const void* A;     // operator: complex64, or packed 16-bit pairs
   const float* rs;   // row scales of the FP16 copy, or null
   double2 *pb, *hr;  // (m + 2) x G partials, m + 2 totals
@@ -226,7 +233,32 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_gmres_run(GArgs a, RunArgs p
   __shared__ double2 s_t;
   __shared__ V s_hv[kF32 ? 258 : 1];  // h in the basis' precision
   __shared__ int s_again, s_done, s_abort;
-  const int n = a.n, G = (int)gridDim.x, b = blockIdx.x;
+  // this block's system and its arrays
+  const int G = p.blocks, b = (int)blockIdx.x % G, sys = p.s0 + (int)blockIdx.x / G;
+  const int n = p.ns ? p.ns[sys] : a.n;
+  const size_t vstr = (size_t)a.nrhs * a.n;  // from one basis vector to the next
+  {
+    const size_t ns = (size_t)sys * a.n;
+    a.b += ns;
+    a.x += ns;
+    a.V += ns;
+    if (kF32) a.Vf += ns;
+    p.pout += ns;
+    a.xf += (size_t)sys * a.ld;
+    a.H += (size_t)sys * a.m * (a.m + 1);
+    a.gv += (size_t)sys * (a.m + 1);
+    p.pb += (size_t)sys * (a.m + 2) * G;
+    p.hr += (size_t)sys * (a.m + 2);
+    p.bar += 2 * sys;
+    a.bnorm += sys;
+    a.hnorm += sys;
+    a.res += sys;
+    a.iters += sys;
+    a.done += sys;
+    if (a.skip) a.skip += sys;
+    if (a.bscale) a.bscale += sys;
+    if (kFmt == 2) p.rs += sys * p.sstride;
+  }
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const bool decides = warp == kRunWarps - 1, chains = warp == kRunWarps - 2;
   // a warp's lanes in the Gram-Schmidt phases: four items, real and imaginary part, a quad each
@@ -239,7 +271,6 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_gmres_run(GArgs a, RunArgs p
   V* sw = sV + (size_t)rmax * p.vcols;
   float* part = reinterpret_cast<float*>(sw + rmax);  // [column range][row][re, im]
   V* gV = kF32 ? reinterpret_cast<V*>(a.Vf) : reinterpret_cast<V*>(a.V);
-  const size_t vstr = (size_t)n;  // one right-hand side: vector c at c n
 
   // this warp's rows and columns of the operator
   const int cwi = warp & (p.cw - 1), rw = warp / p.cw, nrw = kRunWarps / p.cw;
@@ -248,7 +279,8 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_gmres_run(GArgs a, RunArgs p
   const int u0 = n32 * cwi / p.cw * 32, len = min(n16, n32 * (cwi + 1) / p.cw * 32) - u0;
   const float4* st0 = reinterpret_cast<const float4*>(smem) + (size_t)warp * p.stages * p.seg;
   const uint32_t ring = sa_u32(st0 + lane);
-  const float4* Ab = reinterpret_cast<const float4*>(p.A) + (size_t)r0 * n16 + u0 + lane;
+  const float4* Ab = reinterpret_cast<const float4*>(p.A) + (size_t)sys * (p.astride / (kFmt == 0 ? 2 : 4)) +
+                     (size_t)r0 * n16 + u0 + lane;
 
   if (tid == 0) {
     s_done = (a.skip && a.skip[0]) ? 1 : 0;
@@ -600,8 +632,10 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_gmres_run(GArgs a, RunArgs p
   if (b == 0 && tid == 0) {
     a.iters[0] = kd;
     a.done[0] = s_done;
-    a.scal[0] = kd;
-    a.scal[1] = 1;
+    if (sys == p.s0) {
+      a.scal[0] = kd;
+      a.scal[1] = 1;
+    }
   }
   if (warp == 0)
     for (int c = b; c < kd; c += G) {

@@ -160,6 +160,8 @@ struct nat_bem_op {
   bool geo_view = false;               // geo belongs to another op of the same mesh
   int64_t bstride = 0;                 // > 0: a batch of operators, RHS s uses L + s bstride
                                        // (and R, Lb likewise); 0: one operator for every RHS
+  const int* batch_n = nullptr;        // a batch: rows of each operator on the device (<= n), or null
+  int share = 1;                       // a batch: solves the caller keeps in flight beside it
   natbem::Workspace* ws = nullptr;     // solver workspace, grown on demand
   bool mc = false;                     // Monte-Carlo op (nat_bem_assemble_mc): n samples
   double mc_area = 0.0;                // Monte-Carlo op: total surface area
