@@ -61,6 +61,7 @@ struct Workspace {
   double2 *pblk = nullptr, *hred = nullptr;                // fused kernel: block partials, totals
   int arn_smem = 0;                                        // fused kernel: dynamic shared bytes
   double2* pbu = nullptr;                                  // multi-RHS fused kernel: unit partials
+  double2* dec = nullptr;                                  // and decisions
   float2* wf = nullptr;                                    // multi-RHS fused kernel: FP32 w
   // captured iteration chunks: key (engine, RHS count, first iteration, count, cap, tol, mode
   // bits: 1 skip flags, 2 accumulate, 4 tolerance relative to ||R g||). The RHS count is part
@@ -1461,20 +1462,23 @@ __global__ void __launch_bounds__(256, 2) k_arnoldi_f32(GArgs a, double2* __rest
 // block streams long coalesced row ranges of V with no per-RHS barrier, and the FP64 pipe stays
 // busy. Per unit and pass: (A) partial dots of its rows for c <= j and ||w||^2 (warp c % 8 per
 // column, lanes over rows, four accumulators), stored per (RHS, column, chunk); barrier; (R)
-// totals over the chunks of each RHS, one thread per (RHS, column), fixed order; barrier; (B)
-// every block takes the decisions for every RHS from the totals (so all blocks agree on the
-// barrier count), then updates its units' rows, and the owner of chunk 0 of an RHS applies
-// its Givens rotation. Same arithmetic and second-pass test as k_arnoldi.
+// block s mod G sums RHS s's chunks, a warp per column, in a fixed order, and takes its decision
+// (||w - V h||, its inverse, second pass or not); barrier; (B) every block reads the decisions (so
+// all agree on the barrier count) and updates its units' rows, while the last warp of block s mod G
+// applies RHS s's Givens rotation; the last RHS to get there advances the iteration. Same
+// arithmetic and second-pass test as k_arnoldi. (With the decisions taken by every block for every
+// RHS, 30 FP64 warp instructions of 76 cycles each, they were 40 us of a 115 us step at 64 RHS.)
 // kF32: the FP32 basis of inner refinement solves (a.Vf, a.wf): the dots and the row updates
 // run in FP32 (lane sums in FP32, unit and chunk totals, Hessenberg column and rotations in
 // FP64), so the loop over the basis uses no FP64 instruction and reads half the bytes. An inner
 // solve stops at a relative residual of 1e-2, far above the FP32 basis' loss of orthogonality.
+// w32: the product already left w as FP32 in a.wf.
 template <bool kF32>
 __global__ void __launch_bounds__(256) k_arnoldi_units(GArgs a, double2* __restrict__ pbu, double2* __restrict__ hr,
-                                                       unsigned* __restrict__ bar, int* __restrict__ err,
-                                                       int unit, int cps) {
+                                                       double2* __restrict__ dec, unsigned* __restrict__ bar,
+                                                       int* __restrict__ err, int unit, int cps, int w32) {
   __shared__ float2 s_hf[256];
-  __shared__ double2 s_h[256];
+  __shared__ double2 s_h[258];
   __shared__ double2 s_acc[256];
   __shared__ double2 s_sn[256];
   __shared__ double s_cs[256];
@@ -1487,8 +1491,17 @@ __global__ void __launch_bounds__(256) k_arnoldi_units(GArgs a, double2* __restr
   const int np = j + 2;
   const size_t ps = (size_t)(a.m + 2);
   const int nunits = a.nrhs * cps;
-  for (int q = threadIdx.x; q < a.nrhs; q += blockDim.x) s_act[q] = a.done[q] ? 0 : 1;
-  __syncthreads();
+  int active = 0;
+  for (int q0 = 0; q0 < a.nrhs; q0 += 256) {
+    const int q = q0 + threadIdx.x;
+    const bool act = q < a.nrhs && !a.done[q];
+    if (q < a.nrhs) s_act[q] = act ? 1 : 0;
+    active += __syncthreads_count(act);
+  }
+  if (!active) {
+    if (b == 0 && threadIdx.x == 0) a.scal[1] = 1;
+    return;
+  }
 
   for (int pass = 0; pass < 2; ++pass) {
     const unsigned char want = pass == 0 ? 1 : 2;
@@ -1498,7 +1511,7 @@ __global__ void __launch_bounds__(256) k_arnoldi_units(GArgs a, double2* __restr
     if constexpr (kF32) {
       // FP32 copy of this block's rows of w = L v_j (the second pass reads the w - V h that
       // the first pass left there)
-      if (pass == 0) {
+      if (pass == 0 && !w32) {
         for (int u = b; u < nunits; u += G) {
           const int s = u / cps, chunk = u % cps;
           if (s_act[s] < want) continue;
@@ -1608,56 +1621,101 @@ __global__ void __launch_bounds__(256) k_arnoldi_units(GArgs a, double2* __restr
     }
     }
     grid_sync(bar, bar + 1, G, err);
-    // (R) totals over the chunks, one thread per (RHS, column)
-    for (int it = b * blockDim.x + threadIdx.x; it < a.nrhs * np; it += G * blockDim.x) {
-      const int s = it / np, c = it % np;
+    // (R) totals over the chunks and the decision of RHS s, by block s mod G
+    for (int s = b; s < a.nrhs; s += G) {
       if (s_act[s] < want) continue;
-      const double2* src = pbu + ((size_t)s * ps + c) * cps;
-      double re = 0.0, im = 0.0;
-      for (int q = 0; q < cps; ++q) {
-        re += src[q].x;
-        im += src[q].y;
+      for (int c = warp; c < np; c += 8) {  // real parts in lanes 0-15, imaginary in 16-31
+        const double* src = reinterpret_cast<const double*>(pbu + ((size_t)s * ps + c) * cps) + (lane >> 4);
+        double v = 0.0;
+        for (int q = lane & 15; q < cps; q += 16) v += src[2 * q];
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if ((lane & 15) == 0) {
+          reinterpret_cast<double*>(s_h + c)[lane >> 4] = v;
+          reinterpret_cast<double*>(hr + (size_t)s * ps + c)[lane >> 4] = v;
+        }
       }
-      hr[(size_t)s * ps + c] = make_double2(re, im);
+      __syncthreads();
+      if (warp == 0) {
+        double t = 0.0;
+        for (int c = lane; c <= j; c += 32) t += cabs2(s_h[c]);
+        t = warp_sum(t);
+        if (lane == 0) {
+          const double wn2 = s_h[j + 1].x;
+          const double hn2 = fmax(wn2 - t, 0.0);
+          const bool again = pass == 0 && !(hn2 > 1e-4 * wn2);
+          const double inv = hn2 > 0.0 ? rsqrt_nr(hn2) : 0.0;
+          dec[s] = make_double2(again ? -1.0 : hn2 * inv, inv);
+        }
+      }
+      __syncthreads();
     }
     grid_sync(bar, bar + 1, G, err);
-    // (B) decisions for every RHS (identical in every block)
-    for (int s = warp; s < a.nrhs; s += 8) {
-      if (s_act[s] < want) continue;
-      const double2* hs = hr + (size_t)s * ps;
-      double t = 0.0;
-      for (int c = lane; c <= j; c += 32) t += cabs2(hs[c]);
-      t = warp_sum(t);
-      if (lane == 0) {
-        const double wn2 = hs[j + 1].x;
-        const double hn2 = fmax(wn2 - t, 0.0);
-        const bool again = pass == 0 && !(hn2 > 1e-4 * wn2);
-        const double inv = hn2 > 0.0 ? rsqrt_nr(hn2) : 0.0;
-        s_hn[s] = again ? -1.0 : hn2 * inv;
-        s_inv[s] = inv;
-      }
-    }
-    __syncthreads();
     for (int s = threadIdx.x; s < a.nrhs; s += blockDim.x)
-      if (s_act[s] >= want && s_hn[s] < 0.0) s_act[s] = 2;
+      if (s_act[s] >= want) {
+        const double2 d = __ldcg(dec + s);
+        s_hn[s] = d.x;
+        s_inv[s] = d.y;
+        if (d.x < 0.0) s_act[s] = 2;
+      }
     __syncthreads();
-    // (B) row updates of each unit, v_{j+1}; chunk 0's owner: Hessenberg column and Givens
+    const bool owner = b < a.nrhs;           // the last warp has rotations to form
+    const int nthr = owner ? 224 : 256;      // threads of the row updates
+    auto upd_sync = [&]() { asm volatile("bar.sync 1, %0;" ::"r"(nthr) : "memory"); };
+    if (owner && warp == 7) {
+      for (int s = b; s < a.nrhs; s += G) {
+        if (s_act[s] < want) continue;
+        const double hn = s_hn[s];
+        const bool last = pass == 1 || s_act[s] == 1;
+        const double2* hs = hr + (size_t)s * ps;
+        const size_t ho = (size_t)s * (a.m + 1);
+        for (int c = lane; c <= j; c += 32) {
+          const double2 h = __ldcg(hs + c);
+          const double2 t = pass == 0 ? h : cadd(a.hcol[ho + c], h);
+          if (!last) a.hcol[ho + c] = t;
+          s_acc[c] = t;
+          if (c < j) {
+            s_cs[c] = a.cs[(size_t)s * a.m + c];
+            s_sn[c] = a.sn[(size_t)s * a.m + c];
+          }
+        }
+        __syncwarp();
+        if (last) {
+          givens_warp(a, s, j, hn, s_acc, s_cs, s_sn, lane);
+          __syncwarp();
+          if (lane == 0) {  // the last RHS of the iteration advances it
+            __threadfence();
+            if (atomicAdd(a.scal + 2, 1) == active - 1) {
+              __threadfence();
+              int all = 1;
+              for (int q = 0; q < a.nrhs; ++q) all &= __ldcg(a.done + q);
+              a.scal[2] = 0;
+              a.scal[0] = j + 1;
+              a.scal[1] = all || j + 1 >= a.maxit;
+            }
+          }
+        }
+        __syncwarp();
+      }
+    } else {
+    // (B) row updates of each unit, v_{j+1}
     for (int u = b; u < nunits; u += G) {
       const int s = u / cps, chunk = u % cps;
       if (s_act[s] < want) continue;
       const double hn = s_hn[s], inv = s_inv[s];
-      const bool last = hn >= 0.0;
+      const bool last = pass == 1 || s_act[s] == 1;
       const double2* hs = hr + (size_t)s * ps;
-      __syncthreads();
-      for (int c = threadIdx.x; c <= j; c += blockDim.x) {
-        s_h[c] = hs[c];
-        if constexpr (kF32) s_hf[c] = make_float2((float)hs[c].x, (float)hs[c].y);
+      upd_sync();
+      for (int c = threadIdx.x; c <= j; c += nthr) {
+        const double2 h = __ldcg(hs + c);
+        s_h[c] = h;
+        if constexpr (kF32) s_hf[c] = make_float2((float)h.x, (float)h.y);
       }
-      __syncthreads();
+      upd_sync();
       const int q0 = chunk * unit, q1 = min(a.n, q0 + unit);
       if constexpr (kF32) {
         const float finv = (float)inv;
-        for (int r = q0 + threadIdx.x; r < q1; r += blockDim.x) {
+        for (int r = q0 + threadIdx.x; r < q1; r += nthr) {
           float2 acc[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f),
                            make_float2(0.f, 0.f)};
           int c = 0;
@@ -1690,7 +1748,7 @@ __global__ void __launch_bounds__(256) k_arnoldi_units(GArgs a, double2* __restr
           }
         }
       } else
-      for (int r = q0 + threadIdx.x; r < q1; r += blockDim.x) {
+      for (int r = q0 + threadIdx.x; r < q1; r += nthr) {
         double2 acc[4] = {make_double2(0.0, 0.0), make_double2(0.0, 0.0), make_double2(0.0, 0.0),
                           make_double2(0.0, 0.0)};
         int c = 0;
@@ -1721,28 +1779,9 @@ __global__ void __launch_bounds__(256) k_arnoldi_units(GArgs a, double2* __restr
           a.xf[(size_t)s * a.ld + r] = make_float2((float)v.x, (float)v.y);
         }
       }
-      if (chunk == 0) {
-        const size_t ho = (size_t)s * (a.m + 1);
-        for (int c = threadIdx.x; c <= j; c += blockDim.x) {
-          const double2 t = pass == 0 ? s_h[c] : cadd(a.hcol[ho + c], s_h[c]);
-          if (!last) a.hcol[ho + c] = t;
-          s_acc[c] = t;
-          if (c < j) {
-            s_cs[c] = a.cs[(size_t)s * a.m + c];
-            s_sn[c] = a.sn[(size_t)s * a.m + c];
-          }
-        }
-        __syncthreads();
-        if (last && warp == 0) givens_warp(a, s, j, hn, s_acc, s_cs, s_sn, lane);
-      }
     }
-  }
-  grid_sync(bar, bar + 1, G, err);  // every Givens update before the flags are read
-  if (b == 0 && threadIdx.x == 0) {
-    int all = 1;
-    for (int q = 0; q < a.nrhs; ++q) all &= a.done[q];
-    a.scal[0] = j + 1;
-    a.scal[1] = all || j + 1 >= a.maxit;
+    }
+    __syncthreads();  // the flags and shared arrays of this pass
   }
 }
 
@@ -2133,6 +2172,7 @@ static nat_bem_status workspace_ensure(nat_bem_op* op, int nrhs, cudaStream_t s)
           most = std::max(most, (size_t)q * (size_t)((n + u - 1) / u));
         }
         take(&ws->pbu, most * (mm + 2));
+        take(&ws->dec, nr);
       }
       take(&ws->wf, (size_t)n * nr);  // FP32 w of inner solves on the FP32 basis
       ws->run_ok = (nrhs == 1 || op->bstride > 0) && !std::getenv("NATBEM_NO_RUN_KERNEL") && run_usable();
@@ -2497,7 +2537,8 @@ static nat_bem_status gemv_bf16(const char* name, const uint32_t* A, int n, int 
 // pout and the FP32 copy a.xf. `bf16` selects the operator copy used for the matvec.
 // w = M x for every RHS with the given engine (x = ws->xf, padded to ld).
 static nat_bem_status matvec(nat_bem_op* op, Workspace* ws, int which, int engine, double2* y,
-                             const int* done, const int* scal, const char* name, cudaStream_t s) {
+                             const int* done, const int* scal, const char* name, cudaStream_t s,
+                             float2* yf = nullptr) {
   const int n = (int)op->n, ld = (int)op->geo.ld, nrhs = ws->nrhs;
   const float2* M = which == 0 ? op->L : op->R;
   switch (engine) {
@@ -2508,7 +2549,7 @@ static nat_bem_status matvec(nat_bem_op* op, Workspace* ws, int which, int engin
                        op->copy_fp16 ? op->row_scale : nullptr, op->bstride > 0 ? n : 0);
     default:
       return product(op, which, engine, ws->xf, nrhs, y, done, scal, ws->tc_scratch, ws->tc_bytes,
-                     ws->tc_err, s);
+                     ws->tc_err, s, yf);
   }
 }
 
@@ -2598,10 +2639,15 @@ static nat_bem_status gmres_run(nat_bem_op* op, Workspace* ws, const GArgs& a, i
   // a capturable (non-legacy) stream and are skipped while per-launch tracing is on.
   static const bool env_off = std::getenv("NATBEM_NO_GRAPHS") != nullptr;
   const bool use_graphs = !env_off && !ws->graphs_off && s != nullptr && !tracing_enabled();
+  // tensor-core products for the multi-RHS kernel's FP32 basis leave w as FP32 at once
+  float2* yf = a.Vf && ws->coop_blocks > 0 && nrhs > kArnUnitsMinRhs && ws->pbu &&
+                       (engine == kEngineTf32 || engine == kEngineBf16 || engine == kEngineFp16)
+                   ? ws->wf
+                   : nullptr;
   auto launch_chunk = [&](int it0, int c) -> nat_bem_status {
     for (int q = 0; q < c; ++q) {
       NB_TRY(matvec(op, ws, 0, engine, ws->w, ws->done, ws->scal,
-                    engine == kEngineGemvCopy ? (op->copy_fp16 ? "gemv_fp16" : "gemv_bf16") : "gemv", s));
+                    engine == kEngineGemvCopy ? (op->copy_fp16 ? "gemv_fp16" : "gemv_bf16") : "gemv", s, yf));
       if (ws->coop_blocks > 0) {
         GArgs ac = a;
         double2* pb = ws->pblk;
@@ -2609,10 +2655,10 @@ static nat_bem_status gmres_run(nat_bem_op* op, Workspace* ws, const GArgs& a, i
         unsigned* bar = ws->gbar;
         int* errp = ws->tc_err;
         if (nrhs > kArnUnitsMinRhs && ws->pbu) {
-          double2* pu = ws->pbu;
+          double2 *pu = ws->pbu, *dec = ws->dec;
           int unit = arnoldi_unit(n, nrhs, ws->units_blocks);
-          int cps = (n + unit - 1) / unit;
-          void* args[] = {&ac, &pu, &hr, &bar, &errp, &unit, &cps};
+          int cps = (n + unit - 1) / unit, w32 = yf != nullptr;
+          void* args[] = {&ac, &pu, &hr, &dec, &bar, &errp, &unit, &cps, &w32};
           const void* kern = ac.Vf ? (const void*)k_arnoldi_units<true> : (const void*)k_arnoldi_units<false>;
           NB_LAUNCH("gmres_arnoldi", s, NB_TRY_CUDA(cudaLaunchCooperativeKernel(kern, dim3(ws->units_blocks), dim3(256), args, 0, s)));
           continue;

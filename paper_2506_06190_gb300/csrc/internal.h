@@ -225,9 +225,10 @@ int gemv_tuned_variant(int64_t n);  // -1 before the autotuner met this size
 // kEngineGemvCopy: the GEMV on the low-precision copy (BF16 or row-scaled FP16, by the op).
 enum Engine { kEngineGemv = 0, kEngineGemvCopy = 1, kEngineFp32 = 2, kEngineTf32 = 3, kEngineBf16 = 4,
               kEngineFp16 = 5 };
+// Yf (tensor-core engines only, else null): the result as complex64 there instead of in Y.
 nat_bem_status product(nat_bem_op* op, int which, int engine, const float2* X, int nrhs,
                        double2* Y, const int* done, const int* scal, void* scratch,
-                       size_t scratch_bytes, int* err, cudaStream_t s);
+                       size_t scratch_bytes, int* err, cudaStream_t s, float2* Yf = nullptr);
 size_t tc_workspace_bytes(int64_t n, int64_t ld, int nrhs, int sms);
 // The FP32-accurate multi-RHS product on tensor cores (three-way BF16 split of L and X) runs for
 // products with L and at least kX6MinRhs RHS once ensure_split has built the split of L.

@@ -687,29 +687,55 @@ __global__ void k_pack_b(const float2* __restrict__ X, int ld, int nrhs, int P, 
   }
 }
 
-// Y[c][row] (complex128, column c at Y + c * n) = the sum of the row tile's partial tiles in K
-// order (the CTAs c_lo..c_hi that covered it, see k_tc_gemm; TM rows per tile), in FP64.
-__global__ void k_tc_reduce(const float* __restrict__ part, int n, int TM, int Ng, int P, int nrhs,
-                            int nkb, int per, int msp, double2* __restrict__ Y,
-                            const int* __restrict__ done, const int* __restrict__ scal,
-                            const float* __restrict__ rs) {
+// Y[c][row] (column c at Y + c * n) = the sum of the row tile's partial tiles in K order (the CTAs
+// c_lo..c_hi that covered it, see k_tc_gemm; TM rows per tile): complex128 summed in FP64, or
+// (kF32) complex64 summed as float-float pairs and rounded once, for the Krylov steps that work in
+// FP32 (the FP64 sums and conversions were 32 of 43 us at 20480 rows x 64 RHS, and 21 MB of
+// writes). Four rows of a tile per thread, column blockIdx.y.
+template <bool kF32>
+__global__ void __launch_bounds__(256)
+k_tc_reduce(const float* __restrict__ part, int n, int TM, int Ng, int P, int nkb, int per, int msp,
+            void* __restrict__ Y, const int* __restrict__ done, const int* __restrict__ scal,
+            const float* __restrict__ rs) {
   if (scal && scal[1]) return;
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;  // over nrhs * n
-  if (i >= (int64_t)nrhs * n) return;
-  const int c = (int)(i / n), row = (int)(i % n);
-  if (done && done[c]) return;
-  const int mt = row / TM, r = row % TM;
-  const int64_t first = (int64_t)mt * nkb, last = first + nkb - 1;
-  const int c_lo = (int)(first / per), c_hi = (int)(last / per);
-  double re = 0.0, im = 0.0;
-  for (int cta = c_lo; cta <= c_hi; ++cta) {
-    const int j = mt - (int)(((int64_t)cta * per) / nkb);  // the segment of this tile in CTA cta
-    const float* p = part + ((size_t)cta * msp + j) * (size_t)Ng * TM;
-    re += p[(size_t)c * TM + r];
-    im += p[(size_t)(P + c) * TM + r];
+  const int c = blockIdx.y, row = (blockIdx.x * blockDim.x + threadIdx.x) * 4;
+  if (row >= n || (done && done[c])) return;
+  const int mt = row / TM, r = row % TM;  // TM is a multiple of 4
+  const int first = mt * nkb, c_lo = first / per, c_hi = (first + nkb - 1) / per;
+  float hi[8], lo[8];
+  double sum[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    hi[q] = lo[q] = 0.f;
+    sum[q] = 0.0;
   }
-  const double sc = rs ? (double)rs[row] : 1.0;  // the FP16 copy's row scale (a power of two)
-  Y[(size_t)c * n + row] = make_double2(re * sc, im * sc);
+  for (int cta = c_lo; cta <= c_hi; ++cta) {
+    const int j = mt - cta * per / nkb;  // the segment of this tile in CTA cta
+    const float* p = part + ((size_t)cta * msp + j) * (size_t)Ng * TM + r;
+    const float4 re = *reinterpret_cast<const float4*>(p + (size_t)c * TM);
+    const float4 im = *reinterpret_cast<const float4*>(p + (size_t)(P + c) * TM);
+    const float v[8] = {re.x, im.x, re.y, im.y, re.z, im.z, re.w, im.w};
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      if (kF32) {  // Knuth's TwoSum
+        const float t = hi[q] + v[q], bb = t - hi[q];
+        lo[q] += (hi[q] - (t - bb)) + (v[q] - bb);
+        hi[q] = t;
+      } else {
+        sum[q] += v[q];
+      }
+    }
+  }
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    if (row + e >= n) break;
+    const float sc = rs ? rs[row + e] : 1.f;  // the FP16 copy's row scale (a power of two)
+    const size_t o = (size_t)c * n + row + e;
+    if (kF32)
+      static_cast<float2*>(Y)[o] = make_float2((hi[2 * e] + lo[2 * e]) * sc, (hi[2 * e + 1] + lo[2 * e + 1]) * sc);
+    else
+      static_cast<double2*>(Y)[o] = make_double2(sum[2 * e] * sc, sum[2 * e + 1] * sc);
+  }
 }
 
 // ------------------------------------------------------------- FP32 CUDA-core complex GEMM
@@ -1286,9 +1312,8 @@ static nat_bem_status product_x6(nat_bem_op* op, const float2* X, int nrhs, doub
   NB_LAUNCH("tc_gemm_x6", s, k_tc_gemm_x6<<<pl.grid, kX6Threads, smem, s>>>(ta[0], ta[1], ta[2], tb[0], tb[1], tb[2], n, nkb,
                                                                           pl.per, pl.msp, Ng, stages, part, err, scal));
   NB_CHECK_LAUNCH();
-  const int64_t tot = (int64_t)nrhs * n;
-  NB_LAUNCH("tc_reduce", s, k_tc_reduce<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(
-      part, n, kTcRows, Ng, P, nrhs, nkb, pl.per, pl.msp, Y, done, scal, nullptr));
+  NB_LAUNCH("tc_reduce", s, k_tc_reduce<false><<<dim3((unsigned)((n + 1023) / 1024), (unsigned)nrhs), 256, 0, s>>>(
+      part, n, kTcRows, Ng, P, nkb, pl.per, pl.msp, Y, done, scal, nullptr));
   NB_CHECK_LAUNCH();
   return NAT_BEM_OK;
 }
@@ -1296,7 +1321,7 @@ static nat_bem_status product_x6(nat_bem_op* op, const float2* X, int nrhs, doub
 static nat_bem_status product_shaped(nat_bem_op* op, int which, int engine, const float2* X, int nrhs,
                                      double2* Y, const int* done, const int* scal, void* scratch,
                                      size_t scratch_bytes, int* err, cudaStream_t s,
-                                     const TcShape* force) {
+                                     const TcShape* force, float2* Yf = nullptr) {
   const int n = (int)op->n, ld = which == 1 ? (int)op->ldr : (int)op->geo.ld;
   const float2* M = which == 0 ? op->L : op->R;
   int dev = 0, sms = 148;
@@ -1407,17 +1432,20 @@ static nat_bem_status product_shaped(nat_bem_op* op, int which, int engine, cons
       NB_LAUNCH("tc_gemm_fp16", s, k_tc_gemm<2, 1><<<pl.grid, kTcThreads, smem, s>>>(ta, tb, n, nkb, pl.per, pl.msp, Ng, sh.stages, part, err, scal));
   }
   NB_CHECK_LAUNCH();
-  const int64_t tot = (int64_t)nrhs * n;
-  NB_LAUNCH("tc_reduce", s, k_tc_reduce<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(
-      part, n, TM, Ng, P, nrhs, nkb, pl.per, pl.msp, Y, done, scal, engine == kEngineFp16 ? op->row_scale : nullptr));
+  const dim3 rgrid((unsigned)((n + 1023) / 1024), (unsigned)nrhs);
+  const float* rs = engine == kEngineFp16 ? op->row_scale : nullptr;
+  if (Yf)
+    NB_LAUNCH("tc_reduce", s, k_tc_reduce<true><<<rgrid, 256, 0, s>>>(part, n, TM, Ng, P, nkb, pl.per, pl.msp, Yf, done, scal, rs));
+  else
+    NB_LAUNCH("tc_reduce", s, k_tc_reduce<false><<<rgrid, 256, 0, s>>>(part, n, TM, Ng, P, nkb, pl.per, pl.msp, Y, done, scal, rs));
   NB_CHECK_LAUNCH();
   return NAT_BEM_OK;
 }
 
 nat_bem_status product(nat_bem_op* op, int which, int engine, const float2* X, int nrhs,
                        double2* Y, const int* done, const int* scal, void* scratch,
-                       size_t scratch_bytes, int* err, cudaStream_t s) {
-  return product_shaped(op, which, engine, X, nrhs, Y, done, scal, scratch, scratch_bytes, err, s, nullptr);
+                       size_t scratch_bytes, int* err, cudaStream_t s, float2* Yf) {
+  return product_shaped(op, which, engine, X, nrhs, Y, done, scal, scratch, scratch_bytes, err, s, nullptr, Yf);
 }
 
 // The tensor-core product's autotuner, run once per (device, size class, Ng, engine) before the
