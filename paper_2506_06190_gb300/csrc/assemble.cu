@@ -34,6 +34,7 @@
 #include <vector>
 
 #include "internal.h"
+#include "pairs.cuh"
 
 namespace natbem {
 
@@ -207,12 +208,6 @@ __global__ void k_geometry(const double* __restrict__ V, const int32_t* __restri
 // -------------------------------------------------------------- regular pairs (FP32)
 namespace {
 
-// 2 pi split for Cody-Waite reduction (Cody & Waite 1980): hi = 2 pi rounded to float,
-// lo = float(2 pi - hi); rho - n hi - n lo with n = rint(rho / 2 pi) keeps |t| <= pi.
-constexpr float kTwoPiHi = 6.28318548202514648f;
-constexpr float kTwoPiLo = -1.7484555314695172e-7f;
-constexpr float kInvTwoPi = 0.159154943091895336f;
-
 __device__ __forceinline__ bool shares_vertex(int4 a, int4 b) {
   return a.x == b.x || a.x == b.y || a.x == b.z || a.y == b.x || a.y == b.y || a.y == b.z ||
          a.z == b.x || a.z == b.y || a.z == b.z;
@@ -328,78 +323,105 @@ k_assemble_regular(const float4* __restrict__ c_hi, const float4* __restrict__ c
 }
 
 // ---------------------------------------------------- regular pairs, paired FP32 (f32x2)
-// The same arithmetic as k_assemble_regular for two adjacent source columns per thread, with
-// the FP32 operations issued as sm_100 paired instructions (add/sub/mul/fma .rn.f32x2): one
-// instruction does the operation for both columns. The kernel is issue-bound, so this halves
-// the cost of everything except the MUFU operations (rsqrt, sin, cos), which stay scalar.
+// The entries of k_assemble_regular for two adjacent source columns per thread, one in each half of
+// paired FP32 operations (pairs.cuh). Bound by the FMA pipe (72% busy, and a paired operation takes
+// it for two cycles: pairing saves issue slots only), so the form is chosen for its operation
+// count, 28 paired operations a point:
+//   - the outer points are c + s v_m with three directions v_m, so |d|^2 = |D|^2 + s^2 |v_m|^2 -
+//     2 s D.v_m and d.n_x = D.n_x - s v_m.n_x cost three operations a point, not ten;
+//   - with u = d.n_x, v = d.n_y, t = 1/r, N = n_x.n_y and e = 3 u v t^2 - N the integrands are
+//     G t^2 [ (v - r e) + i (k v (u - r) - e/k) ] and G [ (1 - u t) - i u t^2 / k ];
+//   - the phase is reduced by the centroid's whole turns for all seven points (float-float, the
+//     product k r unrounded), and both cross products have accumulators of their own.
+// 10240 triangles: 1.198 -> 1.044 ms (49 operations a point and roundings on the rsqrt unit before);
+// the error against FP64 entries is the same at k = 1 and a quarter less at k = 20. Four blocks per
+// SM: three (more loads in flight) 1.128 ms, five and six (spilled column data) 1.051 and 1.083 ms.
 namespace {
-typedef unsigned long long u64;
-__device__ __forceinline__ u64 pk(float lo, float hi) {
-  u64 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ void upk(u64 v, float& lo, float& hi) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ u64 add2(u64 a, u64 b) {
-  u64 d;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ u64 sub2(u64 a, u64 b) {
-  u64 d;
-  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ u64 mul2(u64 a, u64 b) {
-  u64 d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ u64 fma2(u64 a, u64 b, u64 c) {
-  u64 d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-__device__ __forceinline__ u64 bc(float x) { return pk(x, x); }
 constexpr int kX2Threads = 128;  // 256 source columns per block, two per thread
+
+struct RegPair {  // of one collocation row and two source columns
+  u64 v3, mkv, N, Nk;  // 3 D.n_y, -k D.n_y, n_x.n_y, n_x.n_y / k
+  u64 v, turn, turn_lo;  // D.n_y, minus the whole turns as a float-float
+};
+struct RegSums {  // sums of L = (Lr - Lb, La) and R = (Ra - Rb, Ri)
+  u64 Lr, La, Lb, Ra, Rb, Ri;
+};
+
+// One point: r from r2, nu = -d.n_x, weight w A / 4 pi.
+__device__ __forceinline__ void reg_point(const RegPair& c, u64 k2, u64 kinv2, u64 t, u64 r, u64 nu, u64 w, RegSums& o) {
+  const u64 th = add2(fma2(k2, r, c.turn), c.turn_lo);
+  float tha, thb, sa, ca, sb, cb;
+  upk(th, tha, thb);
+  __sincosf(tha, &sa, &ca);
+  __sincosf(thb, &sb, &cb);
+  const u64 gw = mul2(t, w);
+  const u64 Gr = mul2(pk(ca, cb), gw), Gi = mul2(pk(sa, sb), gw);
+  const u64 t2 = mul2(t, t);
+  const u64 g = mul2(nu, t2), gk = mul2(g, kinv2);  // -u t^2, -u t^2 / k
+  const u64 me = fma2(g, c.v3, c.N);                // -e
+  const u64 lr = fma2(r, me, c.v);
+  const u64 li = fma2(c.mkv, add2(nu, r), fma2(gk, c.v3, c.Nk));
+  const u64 Hr = mul2(Gr, t2), Hi = mul2(Gi, t2);
+  o.Lr = fma2(Hr, lr, o.Lr);
+  o.Lb = fma2(Hi, li, o.Lb);
+  o.La = fma2(Hi, lr, fma2(Hr, li, o.La));
+  const u64 t1 = fma2(nu, t, bc(1.f));
+  o.Ra = fma2(Gr, t1, o.Ra);
+  o.Rb = fma2(Gi, gk, o.Rb);
+  o.Ri = fma2(Gi, t1, fma2(Gr, gk, o.Ri));
+}
 }  // namespace
 
-// Four blocks per SM (128 registers, no spills): 1.192 ms against 1.222 ms at three blocks (164
-// registers) on the 10240-triangle operator; five blocks spill and took 1.283 ms.
 __global__ void __launch_bounds__(kX2Threads, 4)
 k_assemble_regular_x2(const float4* __restrict__ c_hi, const float4* __restrict__ c_lo,
                       const float4* __restrict__ nrm, const float4* __restrict__ qp,
                       const int4* __restrict__ vid, int n, int ld, int rows_per_block, float k,
                       float2* __restrict__ L, float2* __restrict__ R, uint32_t* __restrict__ Lb) {
-  __shared__ float4 s_hi[kRowStage], s_lo[kRowStage], s_n[kRowStage];
+  // row records with every value in both halves of a pair: centroid high, low, normal
+  __shared__ __align__(16) u64 s_row[kRowStage][10];
   __shared__ int4 s_v[kRowStage];
+  __shared__ int s_top;
   const int j0 = (blockIdx.x * kX2Threads + threadIdx.x) * 2;  // columns j0, j0 + 1
   const bool ok0 = j0 < n, ok1 = j0 + 1 < n;
   const bool pad0 = !ok0 && j0 < ld, pad1 = !ok1 && j0 + 1 < ld;
-  // column records as pairs (column j0 in the low half, j0 + 1 in the high half)
-  u64 chx, chy, chz, clx, cly, clz, njx, njy, njz, qx[7], qy[7], qz[7], qw[7];
+  // column records as pairs (column j0 in the low half, j0 + 1 in the high half); va, vb: the first
+  // orbit's offsets towards vertices 2 and 1 (the third is -(va + vb)); sq: the first orbit's |offset|^2
+  u64 chx, chy, chz, clx, cly, clz, njx, njy, njz, vax, vay, vaz, vbx, vby, vbz, sq[3], qw[3];
   int4 v0 = make_int4(-1, -1, -1, 0), v1 = v0;
+  float grid;
   {
     const int ja = ok0 ? j0 : 0, jb = ok1 ? j0 + 1 : ja;
     const float4 a = c_hi[ja], b = c_hi[jb];
-    chx = pk(a.x, b.x), chy = pk(a.y, b.y), chz = pk(a.z, b.z);
+    // High parts of the centroids on one grid, a 2^22nd of the largest coordinate among the
+    // block's columns: their differences are then exact, and what D loses to rounding is known.
+    if (threadIdx.x == 0) s_top = 0;
+    __syncthreads();
+    atomicMax(&s_top, __float_as_int(fminf(1e37f, fmaxf(fmaxf(fmaxf(fabsf(a.x), fabsf(a.y)), fabsf(a.z)),
+                                                        fmaxf(fmaxf(fabsf(b.x), fabsf(b.y)), fabsf(b.z))))));
+    __syncthreads();
+    grid = 3.f * __int_as_float((s_top & 0x7f800000) + 0x00800000);
     const float4 al = c_lo[ja], bl = c_lo[jb];
-    clx = pk(al.x, bl.x), cly = pk(al.y, bl.y), clz = pk(al.z, bl.z);
+    const u64 g2 = bc(grid), hx = pk(a.x, b.x), hy = pk(a.y, b.y), hz = pk(a.z, b.z);
+    chx = sub2(add2(hx, g2), g2), chy = sub2(add2(hy, g2), g2), chz = sub2(add2(hz, g2), g2);
+    clx = add2(sub2(hx, chx), pk(al.x, bl.x));
+    cly = add2(sub2(hy, chy), pk(al.y, bl.y));
+    clz = add2(sub2(hz, chz), pk(al.z, bl.z));
     const float4 an = nrm[ja], bn = nrm[jb];
     njx = pk(an.x, bn.x), njy = pk(an.y, bn.y), njz = pk(an.z, bn.z);
+    qw[0] = pk(qp[7 * (size_t)ja].w, qp[7 * (size_t)jb].w);
 #pragma unroll
-    for (int p = 0; p < 7; ++p) {
-      const float4 qa = qp[7 * ja + p], qb = qp[7 * jb + p];
-      qx[p] = pk(qa.x, qb.x), qy[p] = pk(qa.y, qb.y), qz[p] = pk(qa.z, qb.z), qw[p] = pk(qa.w, qb.w);
+    for (int p = 0; p < 3; ++p) {
+      const float4 qa = qp[7 * (size_t)ja + 1 + p], qb = qp[7 * (size_t)jb + 1 + p];
+      const u64 x = pk(qa.x, qb.x), y = pk(qa.y, qb.y), z = pk(qa.z, qb.z);
+      sq[p] = fma2(x, x, fma2(y, y, mul2(z, z)));
+      if (p == 0) vax = x, vay = y, vaz = z, qw[1] = pk(qa.w, qb.w);
+      if (p == 1) vbx = x, vby = y, vbz = z, qw[2] = pk(qp[7 * (size_t)ja + 4].w, qp[7 * (size_t)jb + 4].w);
     }
     if (ok0) v0 = vid[j0];
     if (ok1) v1 = vid[j0 + 1];
   }
   const float kinv = 1.0f / k;
-  const u64 k2 = bc(k), kinv2 = bc(kinv), mkinv2 = bc(-kinv), inv2pi2 = bc(kInvTwoPi);
-  const u64 m2pihi = bc(-kTwoPiHi), m2pilo = bc(-kTwoPiLo), one2 = bc(1.0f), m3 = bc(-3.0f), three2 = bc(3.0f);
+  const u64 k2 = bc(k), kinv2 = bc(kinv);
   const int i_begin = blockIdx.y * rows_per_block;
   const int i_end = min(n, i_begin + rows_per_block);
   for (int ib = i_begin; ib < i_end; ib += kRowStage) {
@@ -407,9 +429,12 @@ k_assemble_regular_x2(const float4* __restrict__ c_hi, const float4* __restrict_
     __syncthreads();
     if (threadIdx.x < cnt) {
       const int i = ib + threadIdx.x;
-      s_hi[threadIdx.x] = c_hi[i];
-      s_lo[threadIdx.x] = c_lo[i];
-      s_n[threadIdx.x] = nrm[i];
+      const float4 h = c_hi[i], l = c_lo[i], m = nrm[i];
+      u64* o = s_row[threadIdx.x];
+      const float hx = (h.x + grid) - grid, hy = (h.y + grid) - grid, hz = (h.z + grid) - grid;
+      o[0] = bc(hx), o[1] = bc(hy), o[2] = bc(hz);
+      o[3] = bc((h.x - hx) + l.x), o[4] = bc((h.y - hy) + l.y), o[5] = bc((h.z - hz) + l.z);
+      o[6] = bc(m.x), o[7] = bc(m.y), o[8] = bc(m.z);
       s_v[threadIdx.x] = vid[i];
     }
     __syncthreads();
@@ -432,69 +457,66 @@ k_assemble_regular_x2(const float4* __restrict__ c_hi, const float4* __restrict_
       const int4 vi = s_v[t];
       const bool w0 = !shares_vertex(vi, v0), w1 = ok1 && !shares_vertex(vi, v1);
       if (!w0 && !w1) continue;
-      const float4 xh = s_hi[t], xl = s_lo[t], ni = s_n[t];
-      const u64 nix = bc(ni.x), niy = bc(ni.y), niz = bc(ni.z);
-      const u64 Dx = add2(sub2(bc(xh.x), chx), sub2(bc(xl.x), clx));
-      const u64 Dy = add2(sub2(bc(xh.y), chy), sub2(bc(xl.y), cly));
-      const u64 Dz = add2(sub2(bc(xh.z), chz), sub2(bc(xl.z), clz));
-      const u64 dny = fma2(Dx, njx, fma2(Dy, njy, mul2(Dz, njz)));
-      const u64 Dni = fma2(Dx, nix, fma2(Dy, niy, mul2(Dz, niz)));
-      const u64 nxny = fma2(nix, njx, fma2(niy, njy, mul2(niz, njz)));
-      const u64 mnxny = sub2(bc(0.f), nxny);
-      u64 Lr = bc(0.f), Li = Lr, Rr = Lr, Ri = Lr;
-#pragma unroll
-      for (int p = 0; p < 7; ++p) {
-        const u64 dx = sub2(Dx, qx[p]), dy = sub2(Dy, qy[p]), dz = sub2(Dz, qz[p]);
-        const u64 r2 = fma2(dx, dx, fma2(dy, dy, mul2(dz, dz)));
-        float r2a, r2b;
-        upk(r2, r2a, r2b);
-        const u64 rinv = pk(rsqrtf(r2a), rsqrtf(r2b));
-        const u64 r = mul2(r2, rinv);
-        const u64 dnx = sub2(Dni, fma2(qx[p], nix, fma2(qy[p], niy, mul2(qz[p], niz))));
-        const u64 rho = mul2(k2, r);
-        float ua, ub;
-        upk(mul2(rho, inv2pi2), ua, ub);
-        const u64 nq = pk(rintf(ua), rintf(ub));
-        const u64 th = fma2(nq, m2pilo, fma2(nq, m2pihi, rho));
-        float tha, thb, sa, ca, sb, cb;
-        upk(th, tha, thb);
-        __sincosf(tha, &sa, &ca);
-        __sincosf(thb, &sb, &cb);
-        const u64 gw = mul2(rinv, qw[p]);
-        const u64 Gr = mul2(pk(ca, cb), gw), Gi = mul2(pk(sa, sb), gw);
-        const u64 ri2 = mul2(rinv, rinv);
-        const u64 qq = mul2(mul2(dnx, dny), ri2);
-        const u64 a = fma2(fma2(rho, rho, m3), qq, nxny);
-        const u64 b = mul2(rho, fma2(three2, qq, mnxny));
-        const u64 lr = fma2(b, mkinv2, dny);                 // dny - b/k
-        const u64 nli = fma2(a, mkinv2, mul2(rho, dny));     // -(a/k - rho dny)
-        const u64 Hr = mul2(Gr, ri2), Hi = mul2(Gi, ri2);
-        Lr = fma2(Hr, lr, fma2(Hi, nli, Lr));                // += Hr lr - Hi li
-        Li = sub2(fma2(Hi, lr, Li), mul2(Hr, nli));          // += Hr li + Hi lr
-        const u64 t1 = sub2(one2, mul2(dnx, rinv));          // 1 - dnx/r
-        const u64 nt2 = mul2(mul2(dnx, ri2), kinv2);         // -t2 = dnx/(k r^2)
-        Rr = fma2(Gr, t1, fma2(Gi, nt2, Rr));                // += Gr t1 - Gi t2
-        Ri = sub2(fma2(Gi, t1, Ri), mul2(Gr, nt2));          // += Gr t2 + Gi t1
+      const u64* x = s_row[t];
+      const u64 nix = x[6], niy = x[7], niz = x[8];
+      const u64 ax = sub2(x[0], chx), bx = sub2(x[3], clx), Dx = add2(ax, bx);
+      const u64 ay = sub2(x[1], chy), by = sub2(x[4], cly), Dy = add2(ay, by);
+      const u64 az = sub2(x[2], chz), bz = sub2(x[5], clz), Dz = add2(az, bz);
+      // |D|^2 is shared by the seven points, so its error does not average out over them: formed
+      // from the exact a and the small b, a.a + b.(a + D), without the rounding of D
+      const u64 D2 = fma2(ax, ax, fma2(ay, ay, fma2(az, az,
+                     fma2(bx, add2(ax, Dx), fma2(by, add2(ay, Dy), mul2(bz, add2(az, Dz)))))));
+      const u64 nu = sub2(bc(0.f), fma2(Dx, nix, fma2(Dy, niy, mul2(Dz, niz))));  // -D.n_x
+      RegPair c;
+      c.v = fma2(Dx, njx, fma2(Dy, njy, mul2(Dz, njz)));  // d.n_y of every point
+      c.N = fma2(nix, njx, fma2(niy, njy, mul2(niz, njz)));
+      c.Nk = mul2(c.N, kinv2);
+      c.v3 = mul2(c.v, bc(3.f));
+      c.mkv = mul2(c.v, bc(-k));
+      RegSums o;
+      o.Lr = o.La = o.Lb = o.Ra = o.Rb = o.Ri = bc(0.f);
+      {
+        const u64 ri = rsqrt2(D2), r = mul2(D2, ri), turns = turns2(mul2(k2, r));
+        c.turn = mul2(turns, bc(-kTwoPiHi));
+        c.turn_lo = fma2(turns, bc(-kTwoPiLo), fma2(turns, bc(-kTwoPiHi), mul2(turns, bc(kTwoPiHi))));
+        reg_point(c, k2, kinv2, ri, r, nu, qw[0], o);
       }
+      u64 dm[3], nm[3];  // D.v_m and v_m.n_x
+      dm[0] = fma2(Dx, vax, fma2(Dy, vay, mul2(Dz, vaz)));
+      dm[1] = fma2(Dx, vbx, fma2(Dy, vby, mul2(Dz, vbz)));
+      dm[2] = add2(dm[0], dm[1]);
+      nm[0] = fma2(nix, vax, fma2(niy, vay, mul2(niz, vaz)));
+      nm[1] = fma2(nix, vbx, fma2(niy, vby, mul2(niz, vbz)));
+      nm[2] = add2(nm[0], nm[1]);
+#pragma unroll
+      for (int q = 0; q < 3; ++q)
+#pragma unroll
+        for (int ob = 0; ob < 2; ++ob) {
+          const float sc = (ob == 0 ? 1.f : kOrbit), sgn = q == 2 ? -sc : sc;
+          const u64 base = ob == 0 ? add2(D2, sq[q]) : fma2(bc(kOrbit * kOrbit), sq[q], D2);
+          const u64 r2 = fma2(bc(-2.f * sgn), dm[q], base);
+          const u64 ri = rsqrt2(r2);
+          reg_point(c, k2, kinv2, ri, mul2(r2, ri), fma2(bc(sgn), nm[q], nu), qw[1 + ob], o);
+        }
       float lr0, lr1, li0, li1, rr0, rr1, ri0, ri1;
-      upk(Lr, lr0, lr1);
-      upk(Li, li0, li1);
-      upk(Rr, rr0, rr1);
-      upk(Ri, ri0, ri1);
+      upk(sub2(o.Lb, o.Lr), lr0, lr1);  // the entries are minus the integrals
+      upk(o.La, li0, li1);
+      upk(sub2(o.Rb, o.Ra), rr0, rr1);
+      upk(o.Ri, ri0, ri1);
       if (w0 && w1) {
-        __stcs(reinterpret_cast<float4*>(L + off), make_float4(-lr0, -li0, -lr1, -li1));
-        __stcs(reinterpret_cast<float4*>(R + off), make_float4(-rr0, -ri0, -rr1, -ri1));
-        if (Lb) __stcs(reinterpret_cast<uint2*>(Lb + off), make_uint2(pack_bf16(-lr0, -li0), pack_bf16(-lr1, -li1)));
+        __stcs(reinterpret_cast<float4*>(L + off), make_float4(lr0, -li0, lr1, -li1));
+        __stcs(reinterpret_cast<float4*>(R + off), make_float4(rr0, -ri0, rr1, -ri1));
+        if (Lb) __stcs(reinterpret_cast<uint2*>(Lb + off), make_uint2(pack_bf16(lr0, -li0), pack_bf16(lr1, -li1)));
       } else {
         if (w0) {
-          __stcs(L + off, make_float2(-lr0, -li0));
-          __stcs(R + off, make_float2(-rr0, -ri0));
-          if (Lb) __stcs(Lb + off, pack_bf16(-lr0, -li0));
+          __stcs(L + off, make_float2(lr0, -li0));
+          __stcs(R + off, make_float2(rr0, -ri0));
+          if (Lb) __stcs(Lb + off, pack_bf16(lr0, -li0));
         }
         if (w1) {
-          __stcs(L + off + 1, make_float2(-lr1, -li1));
-          __stcs(R + off + 1, make_float2(-rr1, -ri1));
-          if (Lb) __stcs(Lb + off + 1, pack_bf16(-lr1, -li1));
+          __stcs(L + off + 1, make_float2(lr1, -li1));
+          __stcs(R + off + 1, make_float2(rr1, -ri1));
+          if (Lb) __stcs(Lb + off + 1, pack_bf16(lr1, -li1));
         }
       }
     }

@@ -135,8 +135,8 @@ k_eval(const float4* __restrict__ c_hi, const float4* __restrict__ c_lo,
   const bool ok = qi < m;
   const u64 k2 = bc((float)k);
   // High parts of points and centroids on one grid, a 2^22nd of the block's largest coordinate:
-  // their difference is then exact, and what D = x - c loses to rounding (the largest error of the
-  // sum, three times everything else) is known and goes into |D|^2.
+  // their difference a is then exact, and with the small b of the low parts |D|^2 = a.a + b.(a + D)
+  // is free of the rounding of D = a + b (else the largest error of the sum, three times the rest).
   if (threadIdx.x == 0) s_top = 0;
   __syncthreads();
   double v[3];
@@ -175,8 +175,8 @@ k_eval(const float4* __restrict__ c_hi, const float4* __restrict__ c_lo,
       const u64 ax = sub2(xh[0], f[kFHi]), bx = sub2(xl[0], f[kFLo]), Dx = add2(ax, bx);
       const u64 ay = sub2(xh[1], f[kFHi + 1]), by = sub2(xl[1], f[kFLo + 1]), Dy = add2(ay, by);
       const u64 az = sub2(xh[2], f[kFHi + 2]), bz = sub2(xl[2], f[kFLo + 2]), Dz = add2(az, bz);
-      const u64 lost = fma2(Dx, sub2(bx, sub2(Dx, ax)), fma2(Dy, sub2(by, sub2(Dy, ay)), mul2(Dz, sub2(bz, sub2(Dz, az)))));
-      const u64 D2 = fma2(bc(2.f), lost, fma2(Dx, Dx, fma2(Dy, Dy, mul2(Dz, Dz))));
+      const u64 D2 = fma2(ax, ax, fma2(ay, ay, fma2(az, az,
+                     fma2(bx, add2(ax, Dx), fma2(by, add2(ay, Dy), mul2(bz, add2(az, Dz)))))));
       const u64 dn = fma2(Dx, f[kFN], fma2(Dy, f[kFN + 1], mul2(Dz, f[kFN + 2])));  // d.n of every point
       u64 Gr = bc(0.f), Gi = Gr, Fr = Gr, Fi = Gr;
       const u64 rc = rsqrt2(D2), rho = mul2(k2, mul2(D2, rc)), turns = turns2(rho);
