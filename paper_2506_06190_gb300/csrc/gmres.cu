@@ -2013,7 +2013,7 @@ int64_t workspace_bytes(int64_t n, int nrhs, const nat_bem_opts& o) {
   return b;
 }
 
-// Pinned host memory for the workspaces' mirrors: slots of one page-locked block per process, so
+// Pinned host memory for the workspaces' mirrors and flags: slots of one page-locked block per process, so
 // that short-lived ops (a batch builds one per mesh) don't allocate and free page-locked memory,
 // which waits for the whole device. A mirror larger than a slot, or with every slot taken, is
 // allocated by itself.
@@ -2023,6 +2023,7 @@ constexpr int kPinSlots = 64;
 std::mutex g_pin_mu;
 char* g_pin_base = nullptr;
 bool g_pin_used[kPinSlots] = {};
+}  // namespace
 
 char* pin_take(size_t bytes) {
   if (bytes <= kPinSlot) {
@@ -2056,7 +2057,6 @@ void pin_give(char* p) {
   }
   cudaFreeHost(p);
 }
-}  // namespace
 
 void workspace_free(Workspace* ws, cudaStream_t s) {
   if (!ws) return;

@@ -219,6 +219,10 @@ nat_bem_status apply_impl(nat_bem_op* op, int which, int engine, const float2* d
 int64_t workspace_bytes(int64_t n, int nrhs, const nat_bem_opts& o);
 int gemv_tuned_variant(int64_t n);  // -1 before the autotuner met this size
 
+// Page-locked host memory (small blocks from a pool), visible to the device; null when there is none.
+char* pin_take(size_t bytes);
+void pin_give(char* p);
+
 // products.cu: Y = M X for nrhs right-hand sides (M = L for which == 0, R for 1).
 // kEngineFp32: FP32 CUDA-core complex GEMM; kEngineTf32 / kEngineBf16: tcgen05 tensor cores
 // on L (TF32) or its BF16 copy, using `scratch` for the packed B and the split-K partials.

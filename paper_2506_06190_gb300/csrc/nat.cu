@@ -23,8 +23,9 @@
 // The weights stay in shared memory for the kernel's lifetime (at most 160 KB) and the biases
 // live in the kernel's parameter space (uniform reads through the constant cache), so HBM only
 // carries the queries, the grid tables (through L2) and the outputs. The tables are half
-// precision (as tiny-cuda-nn stores its grid parameters); a dense level is laid out so that the
-// four vertices of a cell face at one z share a 32-byte sector.
+// precision (as tiny-cuda-nn stores its grid parameters) and laid out when the field is created so
+// that the four vertices of a cell face at one z share a 32-byte sector, hashed levels as well: a
+// level costs a query two loads from two sectors, where a hashed one took eight of each.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -55,6 +56,13 @@ __host__ __device__ constexpr uint32_t nat_smem_bytes(int k0, int n16, int group
 __host__ __device__ constexpr int nat_k0(int d) { return (16 + 12 * (d - 3) + 15) / 16; }  // layer-0 K steps
 constexpr uint32_t kPrime1 = 2654435761u, kPrime2 = 805459861u;
 
+// Where a level's quads start (8-byte units); of 4: the size of all, 9.8 MB.
+__host__ __device__ constexpr int nat_level_units(int lvl) {
+  int u = 0;
+  for (int l = 0; l < lvl; ++l) u += 4 * (8 << l) * (8 << l) * ((8 << l) + 1);
+  return u;
+}
+
 struct NatBias {
   float b[(kNatHidden + 1) * kNatWidth];  // hidden layers 128 each, then the output layer
 };
@@ -64,15 +72,14 @@ struct NatBias {
 struct nat_field {
   int32_t n_cond = 0, n_out = 0, n16 = 0, table_log2 = 0;
   uint2* tables = nullptr;      // the four levels in half precision (4 features = 8 bytes per
-                                // vertex): a dense level as quads of the (i, j), (i+1, j), (i, j+1),
-                                // (i+1, j+1) vertices at each z (32 bytes, one sector); a hashed
-                                // level as its rows
-  int64_t level_off[4] = {0, 0, 0, 0};  // in 8-byte units, multiples of 4
+                                // vertex) as quads of the (i, j), (i+1, j), (i, j+1), (i+1, j+1)
+                                // vertices at each z (32 bytes, one sector), hashed levels too
   uint16_t* weights = nullptr;  // BF16 [out][in]: 4 x 128 x 128, then n16 x 128 (rows >= n_out zero)
   natbem::NatBias bias{};       // host copy, passed by value to the kernel
   int device = 0;
   cudaStream_t stream = nullptr;
-  int* err = nullptr;           // bounded-wait failures
+  int* err = nullptr;           // bounded-wait failures: a page-locked word the kernel sets and the
+                                // host reads after its wait for the stream, zero between calls
   // host buffers: upload and download streams, created on first use
   cudaStream_t up = nullptr, down = nullptr;
 };
@@ -136,6 +143,11 @@ __device__ __forceinline__ bool nat_bar_wait(uint32_t bar, uint32_t parity) {
     }
   }
   return false;
+}
+
+// 16 bytes from global to shared memory, asynchronously.
+__device__ __forceinline__ void nat_cp16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(nat_smem_u32(dst)), "l"(src) : "memory");
 }
 
 // Barriers of one group of four warps (named barriers 1 and 2; 0 is __syncthreads).
@@ -228,34 +240,25 @@ __device__ __forceinline__ void nat_cell(int lvl, const float (&xv)[D], int (&i0
   }
 }
 
-// Requests the eight corner rows of level lvl. dense_mask bit lvl: the level is stored densely
-// (the quads at z = k and z = k + 1: four 16-byte loads from two 32-byte sectors), else hashed.
+// One quad: 32 bytes, one sector, in one load.
+__device__ __forceinline__ void nat_ld_quad(const uint4* p, uint4& a, uint4& b) {
+  asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
+      : "l"(p));
+}
+
+// Requests the eight corner rows of level lvl: the quads at z = k and z = k + 1.
 template <int D>
-__device__ __forceinline__ void nat_fetch(int lvl, const float (&xv)[D], const uint2* __restrict__ tables,
-                                          const int (&offs)[4], uint32_t hmask, int dense_mask, NatRows& rows) {
+__device__ __forceinline__ void nat_fetch(int lvl, const float (&xv)[D], const uint2* __restrict__ tables, NatRows& rows) {
   const int N = 8 << lvl;
   int i0[3];
   float w1[3];
   nat_cell<D>(lvl, xv, i0, w1);
-  if (dense_mask & (1 << lvl)) {
-    const uint4* tq = reinterpret_cast<const uint4*>(tables + offs[lvl]);
-    const uint32_t q0 = (uint32_t)i0[0] + (uint32_t)N * ((uint32_t)i0[1] + (uint32_t)N * (uint32_t)i0[2]);
-    const uint32_t q1 = q0 + (uint32_t)(N * N);
-    rows.r[0] = __ldg(tq + 2 * q0);
-    rows.r[1] = __ldg(tq + 2 * q0 + 1);
-    rows.r[2] = __ldg(tq + 2 * q1);
-    rows.r[3] = __ldg(tq + 2 * q1 + 1);
-  } else {
-    const uint2* tl = tables + offs[lvl];
-    const uint32_t hx[2] = {(uint32_t)i0[0], (uint32_t)i0[0] + 1u};
-    const uint32_t hy[2] = {(uint32_t)i0[1] * kPrime1, ((uint32_t)i0[1] + 1u) * kPrime1};
-    const uint32_t hz[2] = {(uint32_t)i0[2] * kPrime2, ((uint32_t)i0[2] + 1u) * kPrime2};
-    uint2 u[8];
-#pragma unroll
-    for (int c = 0; c < 8; ++c) u[c] = __ldg(tl + ((hx[c & 1] ^ hy[(c >> 1) & 1] ^ hz[c >> 2]) & hmask));
-#pragma unroll
-    for (int c = 0; c < 4; ++c) rows.r[c] = make_uint4(u[2 * c].x, u[2 * c].y, u[2 * c + 1].x, u[2 * c + 1].y);
-  }
+  const uint4* tq = reinterpret_cast<const uint4*>(tables + nat_level_units(lvl));
+  const uint32_t q0 = (uint32_t)i0[0] + (uint32_t)N * ((uint32_t)i0[1] + (uint32_t)N * (uint32_t)i0[2]);
+  const uint32_t q1 = q0 + (uint32_t)(N * N);
+  nat_ld_quad(tq + 2 * q0, rows.r[0], rows.r[1]);
+  nat_ld_quad(tq + 2 * q1, rows.r[2], rows.r[3]);
 }
 
 // The four trilinear features of level lvl from its fetched rows, as two BF16 pairs.
@@ -315,9 +318,8 @@ __device__ __forceinline__ void nat_store_row(const uint32_t (&pk)[8 * K0], int6
 // G groups of four warps per block, each with its own 128-query tile.
 template <int D, int G>
 __global__ void __launch_bounds__(G * 128, 1)
-k_nat_forward(const float* __restrict__ x, int64_t n, const uint2* __restrict__ tables, int off1, int off2,
-              int off3, int log2, int dense_mask, const uint16_t* __restrict__ weights, int n_out, int n16,
-              float* __restrict__ out, int* __restrict__ err, const __grid_constant__ NatBias P) {
+k_nat_forward(const float* __restrict__ x, int64_t n, const uint2* __restrict__ tables,
+              const uint16_t* __restrict__ weights, int n_out, int n16, float* __restrict__ out, int* __restrict__ err, const __grid_constant__ NatBias P) {
   constexpr int K0 = nat_k0(D);
   constexpr uint32_t kW0 = nat_w0_bytes(K0);
   extern __shared__ uint8_t nat_raw[];
@@ -331,21 +333,30 @@ k_nat_forward(const float* __restrict__ x, int64_t n, const uint2* __restrict__ 
   const int g = threadIdx.x >> 7, t = threadIdx.x & 127, warp = threadIdx.x >> 5;
   uint8_t* sA = sA0 + g * kNatTile;
 
+  // the first tile's rows are requested before the weights: both latencies overlap
+  const int64_t tstride = (int64_t)gridDim.x * G;
+  int64_t tile = (int64_t)g * gridDim.x + blockIdx.x;
+  float xn[D], xnn[D];  // inputs of tiles i + 1 and i + 2
+  NatRows rb[2];        // requested rows of the levels nat_finish uses next (level l in rb[l & 1])
+  NatRows r2, r3;
+  nat_load_x<D>(x, tile * 128 + t, n, xnn);
+  nat_fetch<D>(0, xnn, tables, rb[0]);
+  nat_fetch<D>(1, xnn, tables, rb[1]);
+  nat_fetch<D>(2, xnn, tables, r2);
+  nat_fetch<D>(3, xnn, tables, r3);
+
   // weights into the swizzled operand layout, once per block
   for (int i = threadIdx.x; i < (int)(kW0 / 16); i += G * 128) {  // layer 0: its K regions only
     const int o = (i >> 3) & 127, c = (i >> 10) * 8 + (i & 7);
-    const uint4 v = *reinterpret_cast<const uint4*>(weights + ((size_t)o * 128 + c * 8));
-    *reinterpret_cast<uint4*>(sW + swz(o, c, 128)) = v;
+    nat_cp16(sW + swz(o, c, 128), weights + ((size_t)o * 128 + c * 8));
   }
   for (int i = threadIdx.x; i < 3 * 128 * 16; i += G * 128) {
     const int l = i >> 11, o = (i >> 4) & 127, c = i & 15;
-    const uint4 v = *reinterpret_cast<const uint4*>(weights + ((size_t)((l + 1) * 128 + o) * 128 + c * 8));
-    *reinterpret_cast<uint4*>(sW + kW0 + l * kNatTile + swz(o, c, 128)) = v;
+    nat_cp16(sW + kW0 + l * kNatTile + swz(o, c, 128), weights + ((size_t)((l + 1) * 128 + o) * 128 + c * 8));
   }
   for (int i = threadIdx.x; i < n16 * 16; i += G * 128) {
     const int o = i >> 4, c = i & 15;
-    const uint4 v = *reinterpret_cast<const uint4*>(weights + ((size_t)(kNatHidden * 128 + o) * 128 + c * 8));
-    *reinterpret_cast<uint4*>(sWout + swz(o, c, n16)) = v;
+    nat_cp16(sWout + swz(o, c, n16), weights + ((size_t)(kNatHidden * 128 + o) * 128 + c * 8));
   }
   if (threadIdx.x == 0) {
 #pragma unroll
@@ -362,6 +373,8 @@ k_nat_forward(const float* __restrict__ x, int64_t n, const uint2* __restrict__ 
                  "r"(kCols));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the weights visible to the tensor cores
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -369,8 +382,6 @@ k_nat_forward(const float* __restrict__ x, int64_t n, const uint2* __restrict__ 
   const uint32_t tlane = tmem + ((uint32_t)((warp & 3) * 32) << 16);      // this warp's lanes
   const uint32_t stage = *tmem_slot + (uint32_t)(G * 128 + g * 8 * K0) + ((uint32_t)((warp & 3) * 32) << 16);
   const uint32_t bar = nat_smem_u32(&bars[g]);
-  const int offs[4] = {0, off1, off2, off3};
-  const uint32_t hmask = (1u << log2) - 1u;
   const uint32_t a0 = nat_smem_u32(sA);
   uint32_t phase = 0;
   bool ok_all = true;
@@ -379,25 +390,18 @@ k_nat_forward(const float* __restrict__ x, int64_t n, const uint2* __restrict__ 
   // group encodes one piece of tile i + 1 into its TMEM staging columns (grid level l for l < 4
   // from rows requested two layers earlier; a share of the positional encoding from layer 1
   // on); the row goes into A once the output layer's MMA has read it.
-  const int64_t tstride = (int64_t)gridDim.x * G;
-  int64_t tile = (int64_t)blockIdx.x * G + g;
-  float xn[D], xnn[D];  // inputs of tiles i + 1 and i + 2
-  NatRows rb[2];        // requested rows of the levels nat_finish uses next (level l in rb[l & 1])
   {
     uint32_t pk[8 * K0];
 #pragma unroll
     for (int i = 0; i < 8 * K0; ++i) pk[i] = 0u;
-    float xv[D];
-    nat_load_x<D>(x, tile * 128 + t, n, xv);
-#pragma unroll
-    for (int lvl = 0; lvl < 4; ++lvl) {
-      nat_fetch<D>(lvl, xv, tables, offs, hmask, dense_mask, rb[0]);
-      nat_finish<D>(lvl, xv, rb[0], pk[2 * lvl], pk[2 * lvl + 1]);
-    }
+    nat_finish<D>(0, xnn, rb[0], pk[0], pk[1]);
+    nat_finish<D>(1, xnn, rb[1], pk[2], pk[3]);
+    nat_finish<D>(2, xnn, r2, pk[4], pk[5]);
+    nat_finish<D>(3, xnn, r3, pk[6], pk[7]);
 #pragma unroll
     for (int d = 3; d < D; ++d) {
       uint32_t o[6];
-      nat_pe_input(xv[d], o);
+      nat_pe_input(xnn[d], o);
 #pragma unroll
       for (int l = 0; l < 6; ++l) pk[8 + (d - 3) * 6 + l] = o[l];
     }
@@ -406,8 +410,8 @@ k_nat_forward(const float* __restrict__ x, int64_t n, const uint2* __restrict__ 
     for (int c = 0; c < 8 * K0; c += 2) nat_tmem_st2(stage + (uint32_t)c, 0u, 0u);  // the padding stays zero
   }
   nat_load_x<D>(x, (tile + tstride) * 128 + t, n, xn);
-  nat_fetch<D>(0, xn, tables, offs, hmask, dense_mask, rb[0]);
-  nat_fetch<D>(1, xn, tables, offs, hmask, dense_mask, rb[1]);
+  nat_fetch<D>(0, xn, tables, rb[0]);
+  nat_fetch<D>(1, xn, tables, rb[1]);
   for (;; tile += tstride) {
     const int64_t q0 = tile * 128;
     if (q0 >= n) break;  // uniform over the group
@@ -446,8 +450,8 @@ k_nat_forward(const float* __restrict__ x, int64_t n, const uint2* __restrict__ 
         uint32_t lo, hi;
         nat_finish<D>(l, xn, rb[l & 1], lo, hi);
         nat_tmem_st2(stage + (uint32_t)(2 * l), lo, hi);
-        if (l < 2) nat_fetch<D>(l + 2, xn, tables, offs, hmask, dense_mask, rb[l & 1]);
-        else nat_fetch<D>(l - 2, xnn, tables, offs, hmask, dense_mask, rb[l & 1]);
+        if (l < 2) nat_fetch<D>(l + 2, xn, tables, rb[l & 1]);
+        else nat_fetch<D>(l - 2, xnn, tables, rb[l & 1]);
       }
       if (l >= 1) {
 #pragma unroll
@@ -466,7 +470,7 @@ k_nat_forward(const float* __restrict__ x, int64_t n, const uint2* __restrict__ 
       ok = group_all(1 + g, ok);
       phase ^= 1u;
       if (!ok) {
-        if (t == 0) atomicOr(err, 1);
+        if (t == 0) *reinterpret_cast<volatile int*>(err) = 1;
         ok_all = false;
         break;
       }
@@ -536,26 +540,23 @@ k_nat_forward(const float* __restrict__ x, int64_t n, const uint2* __restrict__ 
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(*tmem_slot), "r"(kCols));
 }
 
-// The caller's FP32 table rows (level after level, min((N+1)^3, 2^log2) rows each) to the
-// half-precision device layout (round to nearest): a dense level as quads, one thread per quad
-// (i, j, k), i, j < N, k <= N; a hashed level row by row.
-__global__ void k_nat_pack(const float4* __restrict__ in, int N, int dense, int64_t rows, uint2* __restrict__ out) {
+// The caller's FP32 table rows of a level (min((N+1)^3, 2^log2) of them, dense or hashed) to the
+// half-precision device layout (round to nearest): one thread per quad (i, j, k), i, j < N,
+// k <= N. Hashing happens here, once, and not at each of a query's eight corners.
+__global__ void k_nat_pack(const float4* __restrict__ in, int N, int dense, uint32_t hmask, uint2* __restrict__ out) {
   const int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   auto h4 = [](float4 v) {
     __half2 a = __floats2half2_rn(v.x, v.y), b = __floats2half2_rn(v.z, v.w);
     return make_uint2(*reinterpret_cast<uint32_t*>(&a), *reinterpret_cast<uint32_t*>(&b));
   };
-  if (!dense) {
-    if (u < rows) out[u] = h4(in[u]);
-    return;
-  }
   const int64_t quads = (int64_t)N * N * (N + 1);
   if (u >= quads) return;
   const int i = (int)(u % N), j = (int)((u / N) % N), k = (int)(u / ((int64_t)N * N));
   const int64_t S1 = N + 1;
 #pragma unroll
   for (int c = 0; c < 4; ++c) {
-    const int64_t r = (i + (c & 1)) + S1 * ((j + (c >> 1)) + S1 * k);
+    const uint32_t ci = (uint32_t)(i + (c & 1)), cj = (uint32_t)(j + (c >> 1)), ck = (uint32_t)k;
+    const int64_t r = dense ? ci + S1 * (cj + S1 * ck) : (int64_t)((ci ^ (cj * kPrime1) ^ (ck * kPrime2)) & hmask);
     out[4 * u + c] = h4(in[r]);
   }
 }
@@ -575,11 +576,6 @@ static nat_bem_status nat_launch_d(const nat_field* f, const float* dx, int64_t 
                                    int sms, bool& attr_done) {
   constexpr int K0 = nat_k0(D);
   const int64_t tiles = (n + 127) / 128;
-  int dense_mask = 0;
-  for (int l = 0; l < 4; ++l) {
-    const int64_t v = (int64_t)(kNatLevels[l] + 1) * (kNatLevels[l] + 1) * (kNatLevels[l] + 1);
-    if (v <= ((int64_t)1 << f->table_log2)) dense_mask |= 1 << l;
-  }
   constexpr bool kThreeFit = nat_smem_bytes(K0, 16, 3) <= kNatSmemLimit;  // three groups possible at all
   if (!attr_done) {
     NB_TRY_CUDA(cudaFuncSetAttribute(k_nat_forward<D, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -589,22 +585,19 @@ static nat_bem_status nat_launch_d(const nat_field* f, const float* dx, int64_t 
                                        (int)kNatSmemLimit));
     attr_done = true;
   }
-  const int off1 = (int)f->level_off[1], off2 = (int)f->level_off[2], off3 = (int)f->level_off[3];
   bool launched = false;
   if constexpr (kThreeFit) {
     if (nat_smem_bytes(K0, f->n16, 3) <= kNatSmemLimit) {
-      const int blocks = (int)std::min<int64_t>((tiles + 2) / 3, (int64_t)sms);
+      const int blocks = (int)std::min<int64_t>(tiles, (int64_t)sms);
       NB_LAUNCH("nat_forward", s, k_nat_forward<D, 3><<<blocks, 384, nat_smem_bytes(K0, f->n16, 3), s>>>(
-          dx, n, f->tables, off1, off2, off3, f->table_log2, dense_mask, f->weights, f->n_out, f->n16, dout,
-          f->err, f->bias));
+          dx, n, f->tables, f->weights, f->n_out, f->n16, dout, f->err, f->bias));
       launched = true;
     }
   }
   if (!launched) {
-    const int blocks = (int)std::min<int64_t>((tiles + 1) / 2, (int64_t)sms);
+    const int blocks = (int)std::min<int64_t>(tiles, (int64_t)sms);
     NB_LAUNCH("nat_forward", s, k_nat_forward<D, 2><<<blocks, 256, nat_smem_bytes(K0, f->n16, 2), s>>>(
-        dx, n, f->tables, off1, off2, off3, f->table_log2, dense_mask, f->weights, f->n_out, f->n16, dout,
-        f->err, f->bias));
+        dx, n, f->tables, f->weights, f->n_out, f->n16, dout, f->err, f->bias));
   }
   NB_CHECK_LAUNCH();
   return NAT_BEM_OK;
@@ -646,6 +639,13 @@ namespace natbem {
 namespace {
 constexpr int64_t kNatChunk = int64_t(1) << 20;  // queries per chunk on the host-buffer path
 
+// The wait flag of the calls that have ended, cleared for the next one.
+int nat_take_err(const nat_field* f) {
+  const int e = *static_cast<volatile int*>(f->err);
+  if (e) *static_cast<volatile int*>(f->err) = 0;
+  return e;
+}
+
 // Host inputs or outputs: chunks of kNatChunk queries in two device buffers each, uploads on
 // one stream, the kernels on the caller's, downloads on another, so that chunk c + 1's upload
 // and chunk c - 1's download run during chunk c's kernel. Queries are independent: the results
@@ -680,7 +680,7 @@ nat_bem_status nat_forward_pipelined(nat_field* f, const float* x, bool xdev, in
     cleanup();
     return st;
   }
-  cudaError_t e = cudaMemsetAsync(f->err, 0, sizeof(int), s);  // this call's bounded-wait flag
+  cudaError_t e = cudaSuccess;
   for (int i = 0; i < 7 && e == cudaSuccess; ++i) e = cudaEventCreateWithFlags(&ev[i], cudaEventDisableTiming);
   // the buffers were allocated on s; the copy streams start after that
   if (e == cudaSuccess) e = cudaEventRecord(ev[0], s);
@@ -722,12 +722,13 @@ nat_bem_status nat_forward_pipelined(nat_field* f, const float* x, bool xdev, in
     // the caller's stream ends after the last download; the buffers are freed on it
     e = cudaEventRecord(ev[0], f->down);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(s, ev[0], 0);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&err, f->err, sizeof(int), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    err = nat_take_err(f);
   } else {
     cudaStreamSynchronize(f->up);
     cudaStreamSynchronize(f->down);
     cudaStreamSynchronize(s);
+    nat_take_err(f);
   }
   if (e != cudaSuccess) {
     set_error(std::string("nat_field_forward: ") + cudaGetErrorString(e));
@@ -765,20 +766,15 @@ nat_bem_status nat_field_create(int32_t n_cond, int32_t n_out, int32_t table_log
     f->table_log2 = table_log2;
     f->stream = s;
     cudaGetDevice(&f->device);
-    // input rows per level, and the device layout's size per level (8-byte units)
-    int64_t rows = 0, units = 0;
-    int64_t in_off[4], in_rows[4];
+    int64_t rows = 0;  // input rows per level
+    int64_t in_off[4];
     bool dense[4];
     for (int l = 0; l < 4; ++l) {
       const int64_t N = kNatLevels[l];
       const int64_t v = (N + 1) * (N + 1) * (N + 1);
       dense[l] = v <= ((int64_t)1 << table_log2);
       in_off[l] = rows;
-      in_rows[l] = std::min<int64_t>(v, (int64_t)1 << table_log2);
-      rows += in_rows[l];
-      f->level_off[l] = units;
-      units += dense[l] ? 4 * N * N * (N + 1) : in_rows[l];
-      units = (units + 3) / 4 * 4;
+      rows += std::min<int64_t>(v, (int64_t)1 << table_log2);
     }
     auto fail = [&](nat_bem_status st) {
       nat_field_destroy(f);
@@ -794,9 +790,12 @@ nat_bem_status nat_field_create(int32_t n_cond, int32_t n_out, int32_t table_log
     float* tw = nullptr;
     nat_bem_status st = to_device(reinterpret_cast<const float4*>(tables), (size_t)rows, s, &din, &tin);
     if (st == NAT_BEM_OK) st = to_device(weights, w_in, s, &dw, &tw);
-    if (st == NAT_BEM_OK) st = dev_alloc_n(&f->tables, (size_t)units, s);
+    if (st == NAT_BEM_OK) st = dev_alloc_n(&f->tables, (size_t)nat_level_units(4), s);
     if (st == NAT_BEM_OK) st = dev_alloc_n(&f->weights, w_rows * 128, s);
-    if (st == NAT_BEM_OK) st = dev_alloc_n(&f->err, 1, s);
+    if (st == NAT_BEM_OK && !(f->err = reinterpret_cast<int*>(pin_take(sizeof(int))))) {
+      set_error("nat_field_create: no page-locked memory for the wait flag");
+      st = NAT_BEM_ECUDA;
+    }
     if (st != NAT_BEM_OK) {
       dev_free(tin, s);
       dev_free(tw, s);
@@ -804,14 +803,14 @@ nat_bem_status nat_field_create(int32_t n_cond, int32_t n_out, int32_t table_log
     }
     for (int l = 0; l < 4; ++l) {
       const int N = kNatLevels[l];
-      const int64_t work = dense[l] ? (int64_t)N * N * (N + 1) : in_rows[l];
-      k_nat_pack<<<(unsigned)((work + 255) / 256), 256, 0, s>>>(din + in_off[l], N, dense[l] ? 1 : 0, in_rows[l],
-                                                                f->tables + f->level_off[l]);
+      const int64_t work = (int64_t)N * N * (N + 1);
+      k_nat_pack<<<(unsigned)((work + 255) / 256), 256, 0, s>>>(din + in_off[l], N, dense[l] ? 1 : 0,
+                                                                (1u << table_log2) - 1u, f->tables + nat_level_units(l));
     }
     const int64_t w_out = (int64_t)w_rows * 128;
     k_nat_weights_bf16<<<(unsigned)((w_out + 255) / 256), 256, 0, s>>>(dw, (int64_t)w_in, w_out, f->weights);
-    cudaError_t e = cudaMemsetAsync(f->err, 0, sizeof(int), s);
-    if (e == cudaSuccess) e = cudaGetLastError();
+    *f->err = 0;
+    cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(f->bias.b, biases, ((size_t)4 * 128 + n_out) * sizeof(float), cudaMemcpyDefault, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -853,17 +852,13 @@ nat_bem_status nat_field_forward(const nat_field* f, const float* x, int64_t n, 
       st = dev_alloc_n(&tout, (size_t)n * f->n_out, s);
       dout = tout;
     }
-    if (st == NAT_BEM_OK && cudaMemsetAsync(f->err, 0, sizeof(int), s) != cudaSuccess) {  // this call's flag
-      set_error("nat_field_forward: could not reset the wait flag");
-      st = NAT_BEM_ECUDA;
-    }
     if (st == NAT_BEM_OK) st = nat_launch(f, dx, n, dout, s);
     int err = 0;
     if (st == NAT_BEM_OK) {
       cudaError_t e = cudaSuccess;
       if (!odev) e = cudaMemcpyAsync(out, tout, (size_t)n * f->n_out * sizeof(float), cudaMemcpyDeviceToHost, s);
-      if (e == cudaSuccess) e = cudaMemcpyAsync(&err, f->err, sizeof(int), cudaMemcpyDeviceToHost, s);
       if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+      err = nat_take_err(f);
       if (e != cudaSuccess) {
         set_error(std::string("nat_field_forward: ") + cudaGetErrorString(e));
         st = NAT_BEM_ECUDA;
@@ -887,7 +882,7 @@ void nat_field_destroy(nat_field* f) {
   if (f->down) cudaStreamDestroy(f->down);
   dev_free(f->tables, f->stream);
   dev_free(f->weights, f->stream);
-  dev_free(f->err, f->stream);
+  pin_give(reinterpret_cast<char*>(f->err));
   delete f;
 }
 
