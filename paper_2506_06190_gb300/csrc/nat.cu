@@ -416,6 +416,7 @@ k_nat_forward(const float* __restrict__ x, int64_t n, const uint2* __restrict__ 
     const int64_t q0 = tile * 128;
     if (q0 >= n) break;  // uniform over the group
     const int64_t q = q0 + t;
+    const bool more = q0 + tstride * 128 < n;  // uniform over the group
     nat_load_x<D>(x, q + 2 * tstride * 128, n, xnn);
 #pragma unroll
     for (int l = 0; l <= kNatHidden; ++l) {
@@ -446,14 +447,14 @@ k_nat_forward(const float* __restrict__ x, int64_t n, const uint2* __restrict__ 
       // earlier into the staging columns, then the request of level l + 2 (of levels 0 and 1 of
       // the tile after it during layers 2 and 3); input d's positional encoding during layer
       // 1 + (d - 3) mod 4
-      if (l < 4) {
+      if (l < 4 && more) {
         uint32_t lo, hi;
         nat_finish<D>(l, xn, rb[l & 1], lo, hi);
         nat_tmem_st2(stage + (uint32_t)(2 * l), lo, hi);
         if (l < 2) nat_fetch<D>(l + 2, xn, tables, rb[l & 1]);
         else nat_fetch<D>(l - 2, xnn, tables, rb[l & 1]);
       }
-      if (l >= 1) {
+      if (l >= 1 && more) {
 #pragma unroll
         for (int d = 3; d < D; ++d)
           if ((d - 3) % 4 == l - 1) {  // input d during layer 1 + (d - 3) mod 4
@@ -517,6 +518,7 @@ k_nat_forward(const float* __restrict__ x, int64_t n, const uint2* __restrict__ 
           }
         }
         // the output layer's MMAs have read A: the next tile's row goes in
+        if (!more) break;
         asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
         uint32_t pk[8 * K0];
 #pragma unroll

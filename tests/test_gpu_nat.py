@@ -217,3 +217,18 @@ def test_host_buffers_pipelined_match_device(nb):
                                         ctypes.c_void_p(oh.ctypes.data), None)
         assert st == nb.NAT_BEM_OK
         assert np.array_equal(oh, ref)                        # device in, host out
+
+
+@pytest.mark.parametrize("n_cond", [2, 8])  # three groups of queries per block, two groups
+def test_tile_edges(nb, n_cond):
+    """Queries are independent: any number of them gives the leading rows of a larger call, bit for
+    bit, at the edges of a tile, of one tile per block and of all groups of a block."""
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    field = nb.NatField.from_params(S.nat_params(n_cond=n_cond, n_out=5, table_log2=13, seed=3))
+    rng = np.random.default_rng(4)
+    x = torch.tensor(rng.random((7 * sms * 128 + 9, 4 + n_cond)), dtype=torch.float32, device="cuda")
+    full = field.forward(x)
+    for n in (1, 127, 128, 129, sms * 128, sms * 128 + 1, 2 * sms * 128 + 1, 3 * sms * 128, 3 * sms * 128 + 1,
+              6 * sms * 128 + 65):
+        assert torch.equal(field.forward(x[:n].contiguous()), full[:n])
