@@ -822,7 +822,7 @@ nat_bem_status nat_bem_reassemble(nat_bem_op* op, double k, void* cuda_stream) {
       return NAT_BEM_EINVAL;
     }
     op->k = k;
-    op->split_ok = false;
+    op->split_of = -1;
     if (op->mc) return mc_assemble_operators(op, (cudaStream_t)cuda_stream);
     if (op->galerkin) return galerkin_assemble_operators(op, (cudaStream_t)cuda_stream);
     NB_TRY(ensure_rules(op->opts.adj_subdiv_levels, op->opts.self_theta_pts));

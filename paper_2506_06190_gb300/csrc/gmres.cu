@@ -2838,7 +2838,7 @@ nat_bem_status apply_impl(nat_bem_op* op, int which, int engine, const float2* d
         return st;
       }
     }
-    if (eng == kEngineFp32 && which == 0 && nrhs >= kX6MinRhs && x6_enabled()) st = ensure_split(op, s);
+    if (eng == kEngineFp32 && which == 0 && nrhs >= kX6MinRhs && x6_enabled()) st = ensure_split(op, 0, s);
     if (eng != kEngineFp32 && which == 0) st = tc_tune(op, eng, nrhs, xpad, y64, scratch, sbytes, err, s);
     if (st == NAT_BEM_OK) st = product(op, which, eng, xpad, nrhs, y64, nullptr, nullptr, scratch, sbytes, err, s);
   }
@@ -2864,8 +2864,6 @@ nat_bem_status solve_impl(nat_bem_op* op, const float2* d_neumann, int nrhs, flo
                           nat_bem_solve_info* info, cudaStream_t s, std::vector<nat_bem_solve_info>* per_rhs,
                           std::vector<int>* per_conv) {
   NB_TRY(workspace_ensure(op, nrhs, s));
-  // the split of L for the FP32-accurate tensor-core products (built outside any capture)
-  if (nrhs >= kX6MinRhs && op->bstride == 0 && x6_enabled()) NB_TRY(ensure_split(op, s));
   Workspace* ws = op->ws;
   const nat_bem_opts& o = op->opts;
   // this solve's bounded-wait flags, barriers and refinement flags
@@ -2881,10 +2879,14 @@ nat_bem_status solve_impl(nat_bem_op* op, const float2* d_neumann, int nrhs, flo
     NB_CHECK_LAUNCH();
     if (nrhs == 1 || op->bstride > 0)  // one RHS, or a batch of operators (one per RHS)
       NB_TRY(gemv("gemv_rhs", op->R, n, ldr, ws->gin, ws->b, nrhs, nullptr, nullptr, s, ws->tc_err, op->bstride));
-    else
+    else {
+      if (nrhs >= kX6RMinRhs && ldr == (int)op->geo.ld && x6_enabled()) NB_TRY(ensure_split(op, 1, s));
       NB_TRY(product(op, 1, kEngineFp32, ws->gin, nrhs, ws->b, nullptr, nullptr, ws->tc_scratch,
                      ws->tc_bytes, ws->tc_err, s));
+    }
   }
+  // the split of L for the FP32-accurate tensor-core products (built outside any capture)
+  if (nrhs >= kX6MinRhs && op->bstride == 0 && x6_enabled()) NB_TRY(ensure_split(op, 0, s));
   std::vector<int> iters(nrhs), done(nrhs), total(nrhs, 0), conv(nrhs, 0);
   std::vector<double> rt(nrhs);
   int tc_err = 0;  // bounded-wait flags of the tensor-core kernels, read at every host sync

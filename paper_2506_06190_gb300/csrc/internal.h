@@ -153,9 +153,9 @@ struct nat_bem_op {
                                        // copy_fp16, packed half2 of the row-scaled entries
   bool copy_fp16 = false;              // mixed FP16: Lb holds L_ij s_i in half precision
   float* row_scale = nullptr;          // mixed FP16: 1 / s_i per row (a power of two)
-  uint16_t* Ls = nullptr;              // FP32-accurate multi-RHS products: L split into three
-                                       // BF16 planes (n x 2 ld each), built on first use
-  bool split_ok = false;               // Ls holds the split of the current L
+  uint16_t* Ls = nullptr;              // FP32-accurate multi-RHS products: L or R split into
+                                       // three BF16 planes (n x 2 ld each), built on first use
+  int split_of = -1;                   // Ls holds the split of the current L (0), R (1) or neither
   bool views = false;                  // L, R and Lb belong to someone else (not freed here)
   bool geo_view = false;               // geo belongs to another op of the same mesh
   int64_t bstride = 0;                 // > 0: a batch of operators, RHS s uses L + s bstride
@@ -235,10 +235,15 @@ nat_bem_status product(nat_bem_op* op, int which, int engine, const float2* X, i
                        size_t scratch_bytes, int* err, cudaStream_t s, float2* Yf = nullptr);
 size_t tc_workspace_bytes(int64_t n, int64_t ld, int nrhs, int sms);
 // The FP32-accurate multi-RHS product on tensor cores (three-way BF16 split of L and X) runs for
-// products with L and at least kX6MinRhs RHS once ensure_split has built the split of L.
+// products with at least kX6MinRhs RHS while Ls holds the split of the matrix (ensure_split; no
+// effect on operators without one). A solve multiplies by R once, so R has to earn the passes
+// that split it, and L again after it when L's split was already there: at 20480 triangles they
+// take 1.26 ms each, the product 0.99 ms for up to 64 RHS, and the CUDA-core product 3.9 ms for 64
+// and about 3 ms for 48.
 constexpr int kX6MinRhs = 8;
+constexpr int kX6RMinRhs = 64;
 bool x6_enabled();
-nat_bem_status ensure_split(nat_bem_op* op, cudaStream_t s);
+nat_bem_status ensure_split(nat_bem_op* op, int which, cudaStream_t s);
 // Picks the tensor-core product's launch shape for this operator size and RHS count by timing
 // the candidates once per size class (outside graph capture); X, Y and scratch are the caller's.
 nat_bem_status tc_tune(nat_bem_op* op, int engine, int nrhs, const float2* X, double2* Y,

@@ -438,24 +438,28 @@ __global__ void k_split3(const float4* __restrict__ a, int64_t count4, __nv_bflo
 }
 
 // B of the x6 product: the layout of k_pack_b's BF16 form, one plane per piece.
+// Two columns of row blockIdx.y per thread.
 __global__ void k_pack_b3(const float2* __restrict__ X, int ld, int nrhs, int P, __nv_bfloat16* __restrict__ B,
                           int64_t plane, const int* __restrict__ scal) {
   if (scal && scal[1]) return;
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;  // over P * ld
-  if (i >= (int64_t)P * ld) return;
-  const int c = (int)(i / ld), j = (int)(i % ld);
-  const float2 x = c < nrhs ? X[(size_t)c * ld + j] : make_float2(0.f, 0.f);
-  const size_t Kt = 2 * (size_t)ld;
-  const float v[4] = {x.x, -x.y, x.y, x.x};
-  const size_t at[4] = {(size_t)c * Kt + 2 * j, (size_t)c * Kt + 2 * j + 1, (size_t)(P + c) * Kt + 2 * j,
-                        (size_t)(P + c) * Kt + 2 * j + 1};
+  const int c = blockIdx.y, j = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
+  if (j >= ld) return;
+  const float4 x = c < nrhs ? *reinterpret_cast<const float4*>(X + (size_t)c * ld + j) : make_float4(0.f, 0.f, 0.f, 0.f);
+  const size_t at = (size_t)c * 2 * ld + 2 * j, to = (size_t)P * 2 * ld;
+  const float v[8] = {x.x, -x.y, x.z, -x.w, x.y, x.x, x.w, x.z};
+  ushort p[3][8];
 #pragma unroll
-  for (int e = 0; e < 4; ++e) {
+  for (int e = 0; e < 8; ++e) {
     __nv_bfloat16 p1, p2, p3;
     split3(v[e], p1, p2, p3);
-    B[at[e]] = p1;
-    B[plane + at[e]] = p2;
-    B[2 * plane + at[e]] = p3;
+    p[0][e] = __bfloat16_as_ushort(p1);
+    p[1][e] = __bfloat16_as_ushort(p2);
+    p[2][e] = __bfloat16_as_ushort(p3);
+  }
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    *reinterpret_cast<ushort4*>(B + q * plane + at) = make_ushort4(p[q][0], p[q][1], p[q][2], p[q][3]);
+    *reinterpret_cast<ushort4*>(B + q * plane + to + at) = make_ushort4(p[q][4], p[q][5], p[q][6], p[q][7]);
   }
 }
 
@@ -657,33 +661,29 @@ k_tc_gemm_x6(const __grid_constant__ CUtensorMap ta1, const __grid_constant__ CU
 // rounded up to 16 (so the epilogue reads whole 32-column TMEM chunks): rows c < P
 // (Re, -Im) pairs, rows P + c (Im, Re) pairs; rows of absent RHS are zero. TF32: FP32 storage;
 // BF16 / FP16: round to nearest (the Krylov vectors have unit norm, inside FP16's range).
+// Two columns of row blockIdx.y per thread, 32-bit indices (a column per thread with 64-bit
+// divisions took 10 us for 64 RHS of 20480 rows).
 template <int kKind>
 __global__ void k_pack_b(const float2* __restrict__ X, int ld, int nrhs, int P, void* __restrict__ B,
                          const int* __restrict__ scal) {
   if (scal && scal[1]) return;
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;  // over P * ld
-  if (i >= (int64_t)P * ld) return;
-  const int c = (int)(i / ld), j = (int)(i % ld);
-  const float2 x = c < nrhs ? X[(size_t)c * ld + j] : make_float2(0.f, 0.f);
-  const size_t Kt = 2 * (size_t)ld;
+  const int c = blockIdx.y, j = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
+  if (j >= ld) return;
+  const float4 x = c < nrhs ? *reinterpret_cast<const float4*>(X + (size_t)c * ld + j) : make_float4(0.f, 0.f, 0.f, 0.f);
+  const size_t at = (size_t)c * 2 * ld + 2 * j, to = (size_t)P * 2 * ld;
+  const float v[8] = {x.x, -x.y, x.z, -x.w, x.y, x.x, x.w, x.z};
   if (kKind == 0) {
     float* b = static_cast<float*>(B);
-    b[(size_t)c * Kt + 2 * j] = x.x;
-    b[(size_t)c * Kt + 2 * j + 1] = -x.y;
-    b[(size_t)(P + c) * Kt + 2 * j] = x.y;
-    b[(size_t)(P + c) * Kt + 2 * j + 1] = x.x;
-  } else if (kKind == 1) {
-    __nv_bfloat16* b = static_cast<__nv_bfloat16*>(B);
-    b[(size_t)c * Kt + 2 * j] = __float2bfloat16_rn(x.x);
-    b[(size_t)c * Kt + 2 * j + 1] = __float2bfloat16_rn(-x.y);
-    b[(size_t)(P + c) * Kt + 2 * j] = __float2bfloat16_rn(x.y);
-    b[(size_t)(P + c) * Kt + 2 * j + 1] = __float2bfloat16_rn(x.x);
+    *reinterpret_cast<float4*>(b + at) = make_float4(v[0], v[1], v[2], v[3]);
+    *reinterpret_cast<float4*>(b + to + at) = make_float4(v[4], v[5], v[6], v[7]);
   } else {
-    __half* b = static_cast<__half*>(B);
-    b[(size_t)c * Kt + 2 * j] = __float2half_rn(x.x);
-    b[(size_t)c * Kt + 2 * j + 1] = __float2half_rn(-x.y);
-    b[(size_t)(P + c) * Kt + 2 * j] = __float2half_rn(x.y);
-    b[(size_t)(P + c) * Kt + 2 * j + 1] = __float2half_rn(x.x);
+    ushort u[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e)
+      u[e] = kKind == 1 ? __bfloat16_as_ushort(__float2bfloat16_rn(v[e])) : __half_as_ushort(__float2half_rn(v[e]));
+    ushort* b = static_cast<ushort*>(B);
+    *reinterpret_cast<ushort4*>(b + at) = make_ushort4(u[0], u[1], u[2], u[3]);
+    *reinterpret_cast<ushort4*>(b + to + at) = make_ushort4(u[4], u[5], u[6], u[7]);
   }
 }
 
@@ -1246,19 +1246,20 @@ static cudaError_t x6_attr() {
   return e;
 }
 
-nat_bem_status ensure_split(nat_bem_op* op, cudaStream_t s) {
-  if (op->views || op->bstride > 0 || !op->L) return NAT_BEM_OK;  // batches run GEMVs
+nat_bem_status ensure_split(nat_bem_op* op, int which, cudaStream_t s) {
+  const float2* M = which == 0 ? op->L : op->R;
+  if (op->views || op->bstride > 0 || !M || (which == 1 && op->ldr != op->geo.ld)) return NAT_BEM_OK;  // batches run GEMVs
   const int64_t Kt = 2 * op->geo.ld;
-  const int64_t count = op->n * Kt;  // floats of L (a multiple of 64)
+  const int64_t count = op->n * Kt;  // floats of M (a multiple of 64)
   if (!op->Ls) NB_TRY(dev_alloc_n(&op->Ls, 3 * (size_t)count, s));
-  if (!op->split_ok) {
+  if (op->split_of != which) {
     int dev = 0, sms = 148;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    NB_LAUNCH("split3", s, k_split3<<<sms * 8, 256, 0, s>>>(reinterpret_cast<const float4*>(op->L), count / 4,
+    NB_LAUNCH("split3", s, k_split3<<<sms * 8, 256, 0, s>>>(reinterpret_cast<const float4*>(M), count / 4,
                                                            reinterpret_cast<__nv_bfloat16*>(op->Ls), count));
     NB_CHECK_LAUNCH();
-    op->split_ok = true;
+    op->split_of = which;
   }
   if (x6_attr() != cudaSuccess) {
     set_error(std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(x6_attr()));
@@ -1267,7 +1268,7 @@ nat_bem_status ensure_split(nat_bem_op* op, cudaStream_t s) {
   return NAT_BEM_OK;
 }
 
-// Y = L X for nrhs <= 64 with the x6 kernel (the caller checked op->split_ok).
+// Y = M X, M = L or R as op->split_of says, for nrhs <= 64 with the x6 kernel (the caller checked op->split_of).
 static nat_bem_status product_x6(nat_bem_op* op, const float2* X, int nrhs, double2* Y, const int* done,
                                  const int* scal, void* scratch, size_t scratch_bytes, int* err, cudaStream_t s,
                                  int sms) {
@@ -1287,8 +1288,7 @@ static nat_bem_status product_x6(nat_bem_op* op, const float2* X, int nrhs, doub
   __nv_bfloat16* B = static_cast<__nv_bfloat16*>(scratch);
   float* part = reinterpret_cast<float*>(static_cast<uint8_t*>(scratch) + bbytes);
   {
-    const int64_t tot = (int64_t)P * ld;
-    NB_LAUNCH("tc_pack", s, k_pack_b3<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(X, ld, nrhs, P, B, (int64_t)bplane, scal));
+    NB_LAUNCH("tc_pack", s, k_pack_b3<<<dim3((unsigned)((ld / 2 + 255) / 256), (unsigned)P), 256, 0, s>>>(X, ld, nrhs, P, B, (int64_t)bplane, scal));
     NB_CHECK_LAUNCH();
   }
   CUtensorMap ta[3], tb[3];
@@ -1327,7 +1327,7 @@ static nat_bem_status product_shaped(nat_bem_op* op, int which, int engine, cons
   int dev = 0, sms = 148;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (engine == kEngineFp32 && which == 0 && nrhs >= kX6MinRhs && op->Ls && op->split_ok && x6_enabled() &&
+  if (engine == kEngineFp32 && nrhs >= kX6MinRhs && op->Ls && op->split_of == which && x6_enabled() &&
       ((uintptr_t)scratch & 255u) == 0) {
     for (int c0 = 0; c0 < nrhs; c0 += 64)  // at most 64 RHS per launch (Ng <= 128 TMEM columns)
       NB_TRY(product_x6(op, X + (size_t)c0 * ld, std::min(64, nrhs - c0), Y + (size_t)c0 * n, done ? done + c0 : nullptr,
@@ -1381,13 +1381,13 @@ static nat_bem_status product_shaped(nat_bem_op* op, int which, int engine, cons
   uint8_t* B = static_cast<uint8_t*>(scratch);
   float* part = reinterpret_cast<float*>(B + round_up(bbytes, 256));
   {
-    const int64_t tot = (int64_t)P * ld;
+    const dim3 pg((unsigned)((ld / 2 + 255) / 256), (unsigned)P);
     if (engine == kEngineTf32)
-      NB_LAUNCH("tc_pack", s, k_pack_b<0><<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(X, ld, nrhs, P, B, scal));
+      NB_LAUNCH("tc_pack", s, k_pack_b<0><<<pg, 256, 0, s>>>(X, ld, nrhs, P, B, scal));
     else if (engine == kEngineBf16)
-      NB_LAUNCH("tc_pack", s, k_pack_b<1><<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(X, ld, nrhs, P, B, scal));
+      NB_LAUNCH("tc_pack", s, k_pack_b<1><<<pg, 256, 0, s>>>(X, ld, nrhs, P, B, scal));
     else
-      NB_LAUNCH("tc_pack", s, k_pack_b<2><<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(X, ld, nrhs, P, B, scal));
+      NB_LAUNCH("tc_pack", s, k_pack_b<2><<<pg, 256, 0, s>>>(X, ld, nrhs, P, B, scal));
     NB_CHECK_LAUNCH();
   }
   CUtensorMap ta, tb;

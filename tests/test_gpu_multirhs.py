@@ -52,3 +52,24 @@ def test_all_columns_zero(nb):
     with nb.Operator.assemble(V, F, 1.0, nb.nat_bem_opts_default(prec=nb.PREC_MIXED_BF16)) as op:
         x, info, st = op.solve(np.zeros((op.n, 9), complex))
         assert st == nb.NAT_BEM_OK and np.all(np.asarray(x) == 0)
+
+
+# The accurate products read a three-way split of R, then of L, from one buffer. Their errors are a
+# few 1e-7 of a column, the solver stops at 1e-6 (floor 4e-6 for single precision): 5e-6 in all.
+@pytest.mark.parametrize("m", [63, 64, 65, 128])
+def test_right_hand_sides_through_the_split_of_r(nb, m):
+    Vs, F = S.ring_sphere(1218)
+    V = S.perturbed_ellipsoid(Vs, 9)
+    g = _neumann(V, F, 2.0, m)
+    with nb.Operator.assemble(V, F, 2.0, nb.nat_bem_opts_default(prec=nb.PREC_MIXED_BF16)) as op:
+        for k in (2.0, 1.5):  # the buffer holds the old L's split when the operator changes
+            if k != 2.0:
+                op.reassemble(k)
+            L, R = op.rows(0, 0, op.n).astype(complex), op.rows(1, 0, op.n).astype(complex)
+            for cols in (slice(0, m), slice(1, 9), slice(0, m)):  # 8 columns need only L's split
+                h = np.ascontiguousarray(g[:, cols])
+                x, info, st = op.solve(h)
+                assert st == nb.NAT_BEM_OK
+                b = R @ h
+                res = np.linalg.norm(L @ np.asarray(x) - b, axis=0)
+                assert np.max(res - 5e-6 * np.linalg.norm(b, axis=0)) <= 0
