@@ -715,13 +715,23 @@ __global__ void __launch_bounds__(256) k_finish(GArgs a, int mode) {
   const int j = a.scal[0];
   const bool active = mode == 0 ? !(a.skip && a.skip[s]) : !a.done[s];
   const int jt = mode == 0 ? 0 : j + 1;
-  double t = 0.0;
-  for (int q = threadIdx.x; q < a.nchunk; q += blockDim.x) t += a.partn[(size_t)q * a.nrhs + s];
-  t = block_sum(t, sh);
-  const double hn = sqrt(t);
+  // the norm and its inverse once per block: every warp's square root and division in FP64 made
+  // this 90 us at 20480 rows x 64 RHS
+  if (threadIdx.x < 32) {
+    double t = 0.0;
+    for (int q = threadIdx.x; q < a.nchunk; q += 32) t += a.partn[(size_t)q * a.nrhs + s];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (threadIdx.x == 0) {
+      sh[0] = sqrt(t);
+      sh[1] = sh[0] > 0.0 ? 1.0 / sh[0] : 0.0;
+    }
+  }
+  __syncthreads();
+  const double hn = sh[0];
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   if (active && hn > 0.0 && r < a.n) {
-    const double inv = 1.0 / hn;
+    const double inv = sh[1];
     const double2 ww = a.w[(size_t)s * a.n + r];
     const double2 v = make_double2(ww.x * inv, ww.y * inv);
     const float2 vf = make_float2((float)v.x, (float)v.y);
@@ -931,7 +941,11 @@ constexpr int kArnPanelBytes = 96 * 1024;
 constexpr int kArnPanelBytesF32 = 48 * 1024;
 constexpr int kArnMaxRhs = 256;
 constexpr int kArnUnitsMinRhs = 4;  // more right-hand sides than this: k_arnoldi_units
-constexpr int kArnUnitsPerSm = 2;   // k_arnoldi_units: blocks per SM (at most)
+// k_arnoldi_units: blocks per SM (at most). Three keep more loads in flight where the basis streams
+// from memory (20480 rows x 64 RHS: 82 -> 70 us a step); with small systems, several of which run
+// side by side in a batch, a grid that leaves room for the others' blocks does better (six
+// requests of up to 6k rows x 48 RHS: 36 ms with two, 43 ms with three).
+constexpr int arn_units_per_sm(int64_t n, int64_t nrhs) { return n * nrhs >= (1 << 20) ? 3 : 2; }
 // mixed refinement: a stalled sweep with every open true residual within this factor of the
 // tolerance ends the solve (the FP32 residual product's rounding floor)
 constexpr double kResidualFloor = 4.0;
@@ -1999,7 +2013,7 @@ int64_t workspace_bytes(int64_t n, int nrhs, const nat_bem_opts& o) {
   b += 8 * nchunk * nrhs;                                            // partial norms
   b += 16 * nrhs * (m + 2) * (256 + 1);   // fused Arnoldi partials (<= 256 blocks) and totals
   if (nrhs > kArnUnitsMinRhs)  // unit partials (about four units per block, <= 160 SMs)
-    b += 16 * (m + 2) * (4 * kArnUnitsPerSm * 160 + nrhs);
+    b += 16 * (m + 2) * (4 * arn_units_per_sm(n, nrhs) * 160 + nrhs);
   b += 8 * n * nrhs;  // FP32 w of inner solves
   if (nrhs > 1) {  // operand and partial tiles of the multi-RHS products
     int dev = 0, sms = 0;
@@ -2160,12 +2174,12 @@ static nat_bem_status workspace_ensure(nat_bem_op* op, int nrhs, cudaStream_t s)
       take(&ws->pblk, nr * (mm + 2) * (size_t)ws->coop_blocks);
       take(&ws->hred, nr * (mm + 2));
       if (nrhs > kArnUnitsMinRhs) {  // the multi-RHS kernel: partials for the largest unit count
-        // its own grid: up to kArnUnitsPerSm blocks per SM (more loads in flight for the
+        // its own grid: two or three blocks per SM (more loads in flight for the
         // streaming dots and row updates; one block per SM kept about a third of the HBM rate)
         int pu32 = 0, pu64 = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pu32, k_arnoldi_units<true>, 256, 0);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pu64, k_arnoldi_units<false>, 256, 0);
-        ws->units_blocks = sms * std::max(1, std::min(kArnUnitsPerSm, std::min(pu32, pu64)));
+        ws->units_blocks = sms * std::max(1, std::min(arn_units_per_sm(n, nrhs), std::min(pu32, pu64)));
         size_t most = 0;
         for (int q = kArnUnitsMinRhs + 1; q <= nrhs; ++q) {
           const int u = arnoldi_unit((int)n, q, ws->units_blocks);

@@ -237,11 +237,11 @@ size_t tc_workspace_bytes(int64_t n, int64_t ld, int nrhs, int sms);
 // The FP32-accurate multi-RHS product on tensor cores (three-way BF16 split of L and X) runs for
 // products with at least kX6MinRhs RHS while Ls holds the split of the matrix (ensure_split; no
 // effect on operators without one). A solve multiplies by R once, so R has to earn the passes
-// that split it, and L again after it when L's split was already there: at 20480 triangles they
-// take 1.26 ms each, the product 0.99 ms for up to 64 RHS, and the CUDA-core product 3.9 ms for 64
-// and about 3 ms for 48.
+// that split it, and L again after it when L's split was already there. At 20480 triangles a
+// split takes 1.28 ms; the product 0.84, 0.94 and 1.00 ms for 32, 48 and 64 RHS, on the CUDA cores
+// 2.5, 4.8 and 4.8 ms.
 constexpr int kX6MinRhs = 8;
-constexpr int kX6RMinRhs = 64;
+constexpr int kX6RMinRhs = 33;
 bool x6_enabled();
 nat_bem_status ensure_split(nat_bem_op* op, int which, cudaStream_t s);
 // Picks the tensor-core product's launch shape for this operator size and RHS count by timing

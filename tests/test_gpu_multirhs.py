@@ -56,7 +56,7 @@ def test_all_columns_zero(nb):
 
 # The accurate products read a three-way split of R, then of L, from one buffer. Their errors are a
 # few 1e-7 of a column, the solver stops at 1e-6 (floor 4e-6 for single precision): 5e-6 in all.
-@pytest.mark.parametrize("m", [63, 64, 65, 128])
+@pytest.mark.parametrize("m", [32, 33, 64, 65, 128])
 def test_right_hand_sides_through_the_split_of_r(nb, m):
     Vs, F = S.ring_sphere(1218)
     V = S.perturbed_ellipsoid(Vs, 9)
