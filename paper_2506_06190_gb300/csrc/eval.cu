@@ -350,17 +350,30 @@ __global__ void k_abs(const float2* __restrict__ v, int64_t count, float* __rest
   if (i < count) out[i] = hypotf(v[i].x, v[i].y);
 }
 
-// out[q, rhs0 + s] = sum over splits of the partials, complex64, column-major (m x nrhs)
-__global__ void k_eval_reduce(const double2* __restrict__ part, int m, int splits, int nr, int stride,
-                              int rhs0, float2* __restrict__ out) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (int64_t)m * nr) return;
-  const int qi = (int)(i / nr), s = (int)(i % nr);
+// out[q, rhs0 + s] = sum over splits of the partials, complex64, column-major (m x nrhs). Bound by
+// the latency of its FP64 chain: eight threads an output, each every eighth split, added in order
+// (one thread took 12-22 us, a tenth of a small field's time).
+__global__ void __launch_bounds__(256)
+k_eval_reduce(const double2* __restrict__ part, int m, int splits, int nr, int stride, int rhs0,
+              float2* __restrict__ out) {
+  __shared__ double2 sh[8][32];
+  const int64_t i = (int64_t)blockIdx.x * 32 + threadIdx.x;
+  const bool ok = i < (int64_t)m * nr;
+  const int qi = ok ? (int)(i / nr) : 0, s = ok ? (int)(i % nr) : 0;
   double re = 0.0, im = 0.0;
-  for (int t = 0; t < splits; ++t) {
+#pragma unroll 4
+  for (int t = threadIdx.y; t < splits; t += 8) {
     const double2 v = part[((size_t)t * m + qi) * stride + s];
     re += v.x;
     im += v.y;
+  }
+  sh[threadIdx.y][threadIdx.x] = make_double2(re, im);
+  __syncthreads();
+  if (threadIdx.y != 0 || !ok) return;
+#pragma unroll
+  for (int y = 1; y < 8; ++y) {
+    re += sh[y][threadIdx.x].x;
+    im += sh[y][threadIdx.x].y;
   }
   out[(size_t)(rhs0 + s) * m + qi] = make_float2((float)re, (float)im);
 }
@@ -459,7 +472,7 @@ static nat_bem_status eval_core(const nat_bem_op* op, const double* d_pts, int64
     NB_LAUNCH("eval", s, eval_launch(src, op->k, nr, grid, s, d_pts, (int)m, d_p, d_g, r0, per_c, part));
     NB_CHECK_LAUNCH();
     const int64_t tot = m * nr;
-    NB_LAUNCH("eval_reduce", s, k_eval_reduce<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(part, (int)m, splits, nr, eval_pass_width(nr), r0, d_out));
+    NB_LAUNCH("eval_reduce", s, k_eval_reduce<<<(unsigned)((tot + 31) / 32), dim3(32, 8), 0, s>>>(part, (int)m, splits, nr, eval_pass_width(nr), r0, d_out));
     NB_CHECK_LAUNCH();
     return NAT_BEM_OK;
   };
@@ -529,7 +542,7 @@ static nat_bem_status far_field_core(const nat_bem_op* op, const double* d_dirs,
       NB_LAUNCH("far_field", s, far_launch_nq<7>(nr, grid, s, *src.g, n, d_dirs, (int)nd, op->k, d_p, d_g, r0, per, part));
     NB_CHECK_LAUNCH();
     const int64_t tot = nd * nr;
-    NB_LAUNCH("eval_reduce", s, k_eval_reduce<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(part, (int)nd, splits, nr, pass_width(nr), r0, d_out));
+    NB_LAUNCH("eval_reduce", s, k_eval_reduce<<<(unsigned)((tot + 31) / 32), dim3(32, 8), 0, s>>>(part, (int)nd, splits, nr, pass_width(nr), r0, d_out));
     NB_CHECK_LAUNCH();
   }
   dev_free(part, s);
@@ -629,7 +642,7 @@ static nat_bem_status eval_noalloc_impl(const nat_bem_op* op, const double* d_pt
     NB_LAUNCH("eval", s, eval_launch(eval_source(op), op->k, nr, grid, s, d_pts, (int)m, d_p, d_g, r0, per, part));
     NB_CHECK_LAUNCH();
     const int64_t tot = m * nr;
-    NB_LAUNCH("eval_reduce", s, k_eval_reduce<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(part, (int)m, splits, nr, eval_pass_width(nr), r0, d_out));
+    NB_LAUNCH("eval_reduce", s, k_eval_reduce<<<(unsigned)((tot + 31) / 32), dim3(32, 8), 0, s>>>(part, (int)m, splits, nr, eval_pass_width(nr), r0, d_out));
     NB_CHECK_LAUNCH();
   }
   return NAT_BEM_OK;
