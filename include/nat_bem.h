@@ -203,6 +203,7 @@ NAT_BEM_API nat_bem_status nat_bem_assemble_mc(const double* pts, const double* 
  * NAT_BEM_EINVAL: NULL arrays, nv or nt < 1, m < 0 or > 2^31 - 1, radius not positive and
  * finite, a triangle index out of range, a degenerate triangle, more than 2^28 grid cells,
  * more samples than cap. NAT_BEM_ENOMEM / NAT_BEM_ECUDA as for nat_bem_assemble.
+ * NAT_BEM_ETIMEOUT: a bounded wait between phases gave up.
  */
 NAT_BEM_API nat_bem_status nat_bem_poisson_sample(const double* verts, int64_t nv, const int32_t* tris,
                                                   int64_t nt, double radius, const double* u, int64_t m,
@@ -319,12 +320,12 @@ NAT_BEM_API nat_bem_status nat_bem_run_batch(nat_bem_job* jobs, int32_t njobs,
  * generation, Sec. 3.4): the jobs' meshes are sorted by size and grouped into buckets of
  * meshes within a factor 2^(1/4) of the bucket's largest triangle count N (at most max_batch
  * meshes, and at most 24 GB of operators per bucket). A bucket is solved as one system of
- * independent operators in lockstep: each mesh's L and R (and BF16 copy) are assembled into
+ * independent operators: each mesh's L and R (and BF16 copy) are assembled into
  * one allocation, padded to N unknowns (identity rows in L, zero rows in R and zero right-hand
- * side entries past the mesh's own n, which leaves its solution unchanged), and every GMRES
- * iteration is one matvec launch over all the bucket's operators and one cooperative Arnoldi
- * launch over all its Krylov spaces (captured in CUDA graphs), each mesh with its own
- * convergence test. Each job's field is then evaluated on its own mesh. Jobs with nrhs > 1
+ * side entries past the mesh's own n, which leaves its solution unchanged), and whole GMRES
+ * runs of the bucket's systems go side by side in cooperative launches, each mesh with its own
+ * blocks and convergence test (systems too large for that: one matvec launch and one Arnoldi
+ * launch per iteration over the whole bucket). Each job's field is then evaluated on its own mesh. Jobs with nrhs > 1
  * are solved one after another through the ordinary path. Results match nat_bem_run_batch's to
  * rounding (summation orders differ with the padded size), within the solver's tolerance.
  *   jobs, njobs, opts: as for nat_bem_run_batch (opts NULL = defaults; NAT_BEM_PREC_MIXED_TF32

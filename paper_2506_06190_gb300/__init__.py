@@ -461,7 +461,7 @@ def nat_bem_run_batch(jobs, opts: Opts | None = None, concurrency: int = 3, stre
 
 def nat_bem_run_batch_fused(jobs, opts: Opts | None = None, max_batch: int = 64, concurrency: int = 4,
                             stream=None):
-    """Fused batch: meshes bucketed by size, each bucket solved in lockstep as one padded system
+    """Fused batch: meshes bucketed by size, each bucket solved as one padded system
     of independent operators (see include/nat_bem.h). Job dicts and results as for
     nat_bem_run_batch."""
     keep, outs = [], []

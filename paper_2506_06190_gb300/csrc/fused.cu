@@ -1,12 +1,13 @@
 // Fused batched solves over meshes of uneven size: instead of one op, stream and launch
 // sequence per job, jobs of similar size are grouped into size buckets and each bucket is
-// solved as one system of B independent operators in lockstep. The bucket's operators are
+// solved as one system of B independent operators. The bucket's operators are
 // padded to its largest triangle count N (rows past a mesh's own n are the identity in L and
 // zero in R, with zero right-hand side entries, so the padded solution is the mesh's own one
-// followed by zeros) and stored back to back in one allocation, N x ld per operator. Every
-// GMRES iteration of the bucket is then one GEMV launch over all B operators (right-hand side
-// s reads operator s) and one cooperative Arnoldi launch over all B Krylov spaces, captured in
-// CUDA graphs, with per-mesh convergence flags so finished meshes drop out of the launches.
+// followed by zeros) and stored back to back in one allocation, N x ld per operator. Whole GMRES
+// runs then go side by side, several systems to a cooperative launch with their own blocks
+// (gmres_run.cuh; share: this worker's part of the device), each ending when it has converged.
+// Systems too large for that take one GEMV launch over all B operators and one cooperative
+// Arnoldi launch over all B Krylov spaces per iteration, with per-mesh convergence flags.
 // Assembly writes each mesh's operators straight into its slice (per-mesh geometry, the same
 // kernels as a single assembly); the field is evaluated per mesh.
 //
@@ -65,7 +66,7 @@ int64_t op_bytes(int64_t N, bool bf16) {
   return N * ld * (16 + (bf16 ? 4 : 0));
 }
 
-// One bucket: assemble every mesh into its slice, pad, solve all in lockstep, evaluate fields.
+// One bucket: assemble every mesh into its slice, pad, solve all, evaluate fields.
 nat_bem_status run_bucket(nat_bem_job* jobs, const Bucket& bk, const nat_bem_opts& o, int share, cudaStream_t s,
                           std::string& first_error) {
   const int B = (int)bk.jobs.size();

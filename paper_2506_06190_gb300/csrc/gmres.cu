@@ -6,8 +6,9 @@
 // one re-orthogonalisation pass (CGS2), the Hessenberg matrix, the complex Givens rotations
 // and the small least-squares solve are FP64.
 //
-// One iteration (all right-hand sides in lockstep, each with its own Krylov space) is two
-// launches: the matvec w = L v_j, then one cooperative kernel (k_arnoldi, or k_arnoldi_units
+// One right-hand side: the whole run in one cooperative launch (gmres_run.cuh) where it fits.
+// Otherwise one iteration (all right-hand sides in lockstep, each with its own Krylov space) is
+// two launches: the matvec w = L v_j, then one cooperative kernel (k_arnoldi, or k_arnoldi_units
 // for many right-hand sides) that does the Gram-Schmidt passes, ||w||, v_{j+1} and the Givens
 // update with grid barriers. Where a cooperative launch cannot hold every block, the same step
 // runs as five kernels (dots, update, dots, update, finish). The iteration index, the per-RHS
@@ -1481,7 +1482,8 @@ __global__ void __launch_bounds__(256, 2) k_arnoldi_f32(GArgs a, double2* __rest
 // all agree on the barrier count) and updates its units' rows, while the last warp of block s mod G
 // applies RHS s's Givens rotation; the last RHS to get there advances the iteration. Same
 // arithmetic and second-pass test as k_arnoldi. (With the decisions taken by every block for every
-// RHS, 30 FP64 warp instructions of 76 cycles each, they were 40 us of a 115 us step at 64 RHS.)
+// RHS, 30 FP64 warp instructions of 76 cycles each, and a third barrier, a step at 20480 rows x 64
+// RHS took 145 us instead of 82; 70 on three blocks per SM.)
 // kF32: the FP32 basis of inner refinement solves (a.Vf, a.wf): the dots and the row updates
 // run in FP32 (lane sums in FP32, unit and chunk totals, Hessenberg column and rotations in
 // FP64), so the loop over the basis uses no FP64 instruction and reads half the bytes. An inner
