@@ -950,22 +950,29 @@ constexpr int arn_units_per_sm(int64_t n, int64_t nrhs) { return n * nrhs >= (1 
 // mixed refinement: a stalled sweep with every open true residual within this factor of the
 // tolerance ends the solve (the FP32 residual product's rounding floor)
 constexpr double kResidualFloor = 4.0;
-// mixed refinement: the inner tolerance of a sweep is inner_tol, loosened once the open true
-// residuals are close to the target: kSweepMargin x (tol / largest open residual) is the
-// contraction still missing (with a margin), rounded down to inner_tol x 2^e, e <= kSweepMaxDoubling
-// (few distinct values, so few captured graphs)
-// (measured on the 10240-triangle interior-source workload, 64 k, 4 in flight, solves/s:
-// 0.15: 136.2, 0.3: 139.1, 0.5: 142.6-143.2, 0.7: 144.4, 1.0: 144.0)
-constexpr double kSweepMargin = 0.7;
-constexpr int kSweepMaxDoubling = 5;
+// mixed refinement: a sweep's inner tolerance is inner_tol, unless the contraction still missing to
+// kSweepTarget x tol is about that or less: then that contraction, rounded down to inner_tol x
+// 2^(e/2), -1 <= e <= 13 (few distinct values, so few captured graphs; the 16-bit copy's own error
+// adds 0.4e-2 of a sweep's start to its end, so tighter ones gain little).
+// Ten bodies of 10240 triangles: 371 iterations in 40 sweeps and errors up to 0.57e-6, against 372 in
+// 39 and up to 1.0e-6 when a sweep was only ever loosened, in whole octaves, towards 0.7 tol; 240
+// solves in buckets of 500 to 8000 triangles: 9224 in 1014 and up to 0.89e-6, against 9094 in 940
+// and up to 1.14e-6 (the batch of 24 takes 2% longer).
+constexpr double kSweepTarget = 0.6;
+// A residual is left alone below this part of tol. Above it, and below tol, another sweep of an
+// iteration or two follows (several right-hand sides: while one is above tol), unless they have
+// stopped contracting: where a sweep ends just under tol or just over it is decided by rounding,
+// and with it whether a solution ends 1.1e-6 or 0.2e-6 off.
+constexpr double kSweepLeave = 0.75;
 
 // The inner tolerance of the next refinement sweep when the largest open relative residual is
 // rho (tol: the outer target; base: the configured inner tolerance).
 inline double sweep_inner_tol(double base, double tol, double rho) {
-  double want = base;
-  const double missing = kSweepMargin * tol / std::max(rho, 1e-300);
-  for (int e = 0; e < kSweepMaxDoubling && 2.0 * want <= missing && 2.0 * want < 1.0; ++e) want *= 2.0;
-  return want;
+  const double missing = kSweepTarget * tol / std::max(rho, 1e-300);
+  if (missing < 0.7 * base) return base;  // 2^(-1/2)
+  int e = (int)std::min(13.0, std::max(-1.0, std::floor(2.0 * std::log2(missing / base))));
+  while (e > 0 && base * std::exp2(0.5 * e) >= 1.0) --e;
+  return base * std::exp2(0.5 * e);
 }
 
 // Rows per work unit of k_arnoldi_units: about four units per block, 64 <= unit <= n.
@@ -2960,15 +2967,16 @@ nat_bem_status solve_impl(nat_bem_op* op, const float2* d_neumann, int nrhs, flo
     std::vector<int> od(nrhs), inner_done(nrhs);
     std::vector<double> prev(nrhs, 1.0);
     // one sweep with the given engine: GMRES on the correction equation (at most a.maxit
-    // iterations), x += d, the true residual and the outer convergence flags
-    auto sweep_once = [&](int eng) -> nat_bem_status {
+    // iterations), x += d, the true residual, and the flags of the right-hand sides at most `leave`
+    auto sweep_once = [&](int eng, double leave) -> nat_bem_status {
       NB_TRY(gmres_run(op, ws, a, eng, 1, d_p, s));
       if (first) {  // the first run started from b = b0: its ||b|| is ||R g||
         NB_TRY_CUDA(cudaMemcpyAsync(ws->b0norm, ws->bnorm, nrhs * sizeof(double), cudaMemcpyDeviceToDevice, s));
         first = false;
       }
-      NB_TRY(matvec(op, ws, 0, accurate, ws->w, nullptr, nullptr, "gemv_resid", s));
-      NB_LAUNCH("ir_residual", s, k_ir_residual<<<vec_grid, kChunk, 0, s>>>(a, ws->b0, ws->outer_done, o.tol));
+      // (systems of a batch that earlier sweeps left alone need no residual any more)
+      NB_TRY(matvec(op, ws, 0, accurate, ws->w, gemv_path ? ws->outer_done : nullptr, nullptr, "gemv_resid", s));
+      NB_LAUNCH("ir_residual", s, k_ir_residual<<<vec_grid, kChunk, 0, s>>>(a, ws->b0, ws->outer_done, leave));
       NB_CHECK_LAUNCH();
       NB_TRY(status_sync(ws, s));  // one host sync per sweep
       status_get(ws, ws->iters, iters.data(), nrhs);
@@ -2989,8 +2997,8 @@ nat_bem_status solve_impl(nat_bem_op* op, const float2* d_neumann, int nrhs, flo
       ++refinements;
       converged = true;
       for (int q = 0; q < nrhs; ++q) {
-        conv[q] = od[q];
-        converged = converged && od[q];
+        conv[q] = od[q] || rt[q] <= o.tol;
+        converged = converged && conv[q];
       }
       return NAT_BEM_OK;
     };
@@ -3004,8 +3012,8 @@ nat_bem_status solve_impl(nat_bem_op* op, const float2* d_neumann, int nrhs, flo
       static const bool fp64_basis = std::getenv("NATBEM_FP64_BASIS") != nullptr;
       const bool fp32_basis =
           !fp64_basis && ws->coop_blocks > 0 && ws->wf && (nrhs <= kArnUnitsMinRhs || ws->pbu != nullptr);
-      // The last sweeps need only the contraction still missing to the outer target, so
-      // their inner tolerance is loosened (sweep_inner_tol); NATBEM_FIXED_INNER_TOL keeps
+      // The last sweeps need only the contraction still missing to the outer target
+      // (sweep_inner_tol); NATBEM_FIXED_INNER_TOL keeps
       // inner_tol for every sweep.
       static const bool fixed_inner = std::getenv("NATBEM_FIXED_INNER_TOL") != nullptr;
       for (int sweep = 0; sweep < o.max_refinements && budget > 0; ++sweep) {
@@ -3015,9 +3023,11 @@ nat_bem_status solve_impl(nat_bem_op* op, const float2* d_neumann, int nrhs, flo
         a.tol = fixed_inner ? o.inner_tol : sweep_inner_tol(o.inner_tol, o.tol, rho);
         a.maxit = std::min(std::min(o.inner_max_iter, budget), ws->m);
         a.Vf = fp32_basis ? reinterpret_cast<float2*>(ws->V) : nullptr;
-        NB_TRY(sweep_once(inner));
+        NB_TRY(sweep_once(inner, kSweepLeave * o.tol));
         a.Vf = nullptr;
-        if (converged) break;
+        bool left = true;  // every right-hand side is below kSweepLeave x tol
+        for (int q = 0; q < nrhs; ++q) left = left && od[q];
+        if (left || (converged && !gemv_path)) break;
         // A sweep that shrank some residual by less than 10x (the low-precision operator's
         // error is comparable to the inner tolerance: high k, ill-conditioned L) or that used
         // up the budget: the rest is solved with the FP32 operator below, with a fresh
@@ -3026,16 +3036,17 @@ nat_bem_status solve_impl(nat_bem_op* op, const float2* d_neumann, int nrhs, flo
         // of the FP32 residual product itself (on modal low-k solves the sweeps contract by
         // 0.01-0.09 down to 1-2e-6 and then by 0.7, and FP32 GMRES on the correction equation
         // ends at the same level): the solve stops there instead.
-        // a stall: some open residual contracted by a factor above 0.1, or above twice the
+        // a stall: some residual above tol contracted by a factor above 0.1, or above twice the
         // inner tolerance of a loosened sweep
         const double stall = std::max(0.1, 2.0 * a.tol);
         double worst = 0.0;
         bool at_floor = true;
         for (int q = 0; q < nrhs; ++q)
-          if (!od[q]) {
+          if (!(converged ? od[q] : conv[q])) {
             worst = std::max(worst, rt[q] / prev[q]);
             at_floor = at_floor && rt[q] <= kResidualFloor * o.tol;
           }
+        if (converged && (worst > stall || budget <= 0)) break;
         if (worst > stall && at_floor) {
           converged = true;
           for (int q = 0; q < nrhs; ++q) conv[q] = 1;
@@ -3058,7 +3069,7 @@ nat_bem_status solve_impl(nat_bem_op* op, const float2* d_neumann, int nrhs, flo
       while (budget > 0) {
         a.bscale = first ? nullptr : ws->b0norm;
         a.maxit = std::min(budget, ws->m);
-        NB_TRY(sweep_once(accurate));
+        NB_TRY(sweep_once(accurate, o.tol));
         converged = true;
         for (int q = 0; q < nrhs; ++q) {
           conv[q] = od[q] || inner_done[q];

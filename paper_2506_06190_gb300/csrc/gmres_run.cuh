@@ -24,7 +24,11 @@
 //     warp, during the next barrier), so all blocks agree on convergence without exchanging it.
 // The arithmetic is that of the two-launch form: FP32 products with compensated FP32 sums, FP64
 // Gram-Schmidt and rotations (FP32 basis for inner refinement solves), the same second-pass
-// test, and sums in a fixed order.
+// test, and sums in a fixed order. A block has more rows than the two-launch form's (64 to 168, there
+// 17 to 80), so on the FP32 basis its sums over rows and over basis vectors are compensated: plain
+// FP32 chains of up to 84 terms left ||w - V h||^2 two to five times further from FP64 sums than
+// that form does, these are as good as FP64 sums of the FP32 vectors. They take 0.4% of a mixed
+// solve (2490 rows: 19.57 -> 19.65 us an iteration).
 //
 // Measured (GB300, one solve in flight, microseconds per iteration, before -> now): see the
 // dispatch in gmres_run.
@@ -179,8 +183,30 @@ __device__ __forceinline__ V run_make(S x, S y) {
   return v;
 }
 
-__device__ __forceinline__ double fma_(double a, double b, double c) { return fma(a, b, c); }
-__device__ __forceinline__ float fma_(float a, float b, float c) { return fmaf(a, b, c); }
+// A running sum of products a b + c d over rows or basis vectors: FP64 as it comes, FP32 compensated.
+template <class S>
+struct RunSum;
+template <>
+struct RunSum<double> {
+  double s = 0.0;
+  __device__ __forceinline__ void add(double a, double b, double c, double d) { s = fma(c, d, fma(a, b, s)); }
+  __device__ __forceinline__ double get() const { return s; }
+  __device__ __forceinline__ double quad() const { return quad_sum(s); }
+};
+template <>
+struct RunSum<float> {
+  float s = 0.f, e = 0.f;
+  __device__ __forceinline__ void add(float a, float b, float c, float d) { kahan_add(s, e, fmaf(a, b, c * d)); }
+  __device__ __forceinline__ float get() const { return s - e; }
+  __device__ __forceinline__ double quad() const {  // over the quad's lanes, as a float pair
+    float hi, lo;
+    two_sum(s, -e, hi, lo);
+#pragma unroll
+    for (int o = 2; o > 0; o >>= 1)
+      df_add(hi, lo, __shfl_xor_sync(0xffffffffu, hi, o), __shfl_xor_sync(0xffffffffu, lo, o));
+    return (double)hi + (double)lo;
+  }
+};
 
 // One warp: column hc[0..j] of the Hessenberg matrix through the earlier rotations, into Hcol, for
 // the least squares, by givens_warp's prefix scan; `top` is its last entry.
@@ -454,9 +480,9 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_gmres_run(GArgs a, RunArgs p
     }
     __syncthreads();
     for (int e = tid; e < 2 * rows; e += kC) {
-      float t = 0.f;
-      for (int q = 0; q < p.cw; ++q) t += part[2 * (q * rmax) + e];
-      S v = (S)t;
+      float t = 0.f, tc = 0.f;  // up to 16 column ranges
+      for (int q = 0; q < p.cw; ++q) kahan_add(t, tc, part[2 * (q * rmax) + e]);
+      S v = (S)(t - tc);
       if (kFmt == 2) v *= (S)p.rs[r0 + (e >> 1)];  // a power of two: exact
       reinterpret_cast<S*>(sw)[e] = v;
     }
@@ -466,17 +492,16 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_gmres_run(GArgs a, RunArgs p
       const int np = j + 2;
       for (int c0 = warp * 4; c0 < np; c0 += kRunWarps * 4) {
         const int c = c0 + item;
-        S acc = 0;
+        RunSum<S> sum;
         if (c < np) {
           const V* v = c > j ? sw : c < p.vcols ? sV + (size_t)c * rmax : gV + c * vstr + r0;
           for (int r = l4; r < rows; r += 4) {
             const V vv = v[r], ww = sw[r];
-            acc = fma_(vv.x, im ? ww.y : ww.x, acc);
-            acc = fma_(vv.y, im ? -ww.x : ww.y, acc);
+            sum.add(vv.x, im ? ww.y : ww.x, vv.y, im ? -ww.x : ww.y);
           }
         }
-        acc = quad_sum(acc);
-        if (l4 == 0 && c < np) __stcg(reinterpret_cast<double*>(p.pb + (size_t)c * G + b) + (im ? 1 : 0), (double)acc);
+        const double acc = sum.quad();
+        if (l4 == 0 && c < np) __stcg(reinterpret_cast<double*>(p.pb + (size_t)c * G + b) + (im ? 1 : 0), acc);
       }
       __syncthreads();
       arrive();
@@ -543,14 +568,14 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_gmres_run(GArgs a, RunArgs p
           const int base = 4 * (warp + q * kRunUpd), row = base + item;
           S acc = 0;
           if (base < rows) {
+            RunSum<S> sum;
             if (row < rows)
               for (int c = l4; c <= j; c += 4) {
                 const V vv = c < p.vcols ? sV[(size_t)c * rmax + row] : gV[c * vstr + r0 + row];
                 const V h = kF32 ? s_hv[c] : reinterpret_cast<const V*>(s_h)[c];
-                acc = fma_(vv.x, im ? h.y : h.x, acc);
-                acc = fma_(vv.y, im ? h.x : -h.y, acc);
+                sum.add(vv.x, im ? h.y : h.x, vv.y, im ? h.x : -h.y);
               }
-            acc = quad_sum(acc);
+            acc = quad_sum(sum.get());
           }
           tsum[q] = acc;
         }
@@ -691,15 +716,14 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_gmres_run(GArgs a, RunArgs p
   // x (+)= V y on the block's rows
   for (int base = 4 * warp; base < rows; base += 4 * kRunWarps) {
     const int row = base + item;
-    S acc = 0;
+    RunSum<S> sum;
     if (row < rows)
       for (int c = l4; c < kd; c += 4) {
         const V vv = c < p.vcols ? sV[(size_t)c * rmax + row] : gV[c * vstr + r0 + row];
         const double2 y = s_hc[c];
-        acc = fma_(vv.x, (S)(im ? y.y : y.x), acc);
-        acc = fma_(vv.y, (S)(im ? y.x : -y.y), acc);
+        sum.add(vv.x, (S)(im ? y.y : y.x), vv.y, (S)(im ? y.x : -y.y));
       }
-    acc = quad_sum(acc);
+    const S acc = quad_sum(sum.get());
     if (row < rows && l4 == 0) {
       const size_t e = 2 * (size_t)(r0 + row) + (im ? 1 : 0);
       double* xe = reinterpret_cast<double*>(a.x) + e;
