@@ -222,6 +222,46 @@ __device__ __forceinline__ uint32_t pack_bf16(float re, float im) {
 constexpr int kRegThreads = 256;  // source columns per block
 constexpr int kRowStage = 64;     // collocation rows staged in shared memory at a time
 
+// Entries (L, R) of a pair with centroid difference D, normals nj (source) and ni (collocation
+// point) and the source's points q: d is formed for every point by itself.
+__device__ __forceinline__ float4 regular_entry(float Dx, float Dy, float Dz, float3 nj, float3 ni,
+                                                const float4* q, float k, float kinv) {
+  const float dny = Dx * nj.x + Dy * nj.y + Dz * nj.z;  // quadrature offsets lie in the plane
+  const float Dni = Dx * ni.x + Dy * ni.y + Dz * ni.z;
+  const float nxny = ni.x * nj.x + ni.y * nj.y + ni.z * nj.z;
+  float Lr = 0.f, Li = 0.f, Rr = 0.f, Ri = 0.f;
+#pragma unroll
+  for (int p = 0; p < 7; ++p) {
+    const float dx = Dx - q[p].x, dy = Dy - q[p].y, dz = Dz - q[p].z;
+    const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+    const float rinv = rsqrtf(r2);
+    const float r = r2 * rinv;
+    const float dnx = Dni - fmaf(q[p].x, ni.x, fmaf(q[p].y, ni.y, q[p].z * ni.z));
+    const float rho = k * r;
+    const float nq = rintf(rho * kInvTwoPi);
+    float th = fmaf(-nq, kTwoPiHi, rho);
+    th = fmaf(-nq, kTwoPiLo, th);
+    float sn, cs;
+    __sincosf(th, &sn, &cs);
+    const float gw = rinv * q[p].w;  // w A / (4 pi r)
+    const float Gr = cs * gw, Gi = sn * gw;
+    const float rinv2 = rinv * rinv;
+    const float qq = dnx * dny * rinv2;
+    const float a = fmaf(fmaf(rho, rho, -3.0f), qq, nxny);
+    const float b = rho * fmaf(3.0f, qq, -nxny);
+    const float lr = fmaf(-b, kinv, dny);
+    const float li = fmaf(a, kinv, -rho * dny);
+    const float Hr = Gr * rinv2, Hi = Gi * rinv2;
+    Lr = fmaf(Hr, lr, fmaf(-Hi, li, Lr));
+    Li = fmaf(Hr, li, fmaf(Hi, lr, Li));
+    const float t1 = fmaf(-dnx, rinv, 1.0f);
+    const float t2 = -dnx * rinv2 * kinv;
+    Rr = fmaf(Gr, t1, fmaf(-Gi, t2, Rr));
+    Ri = fmaf(Gr, t2, fmaf(Gi, t1, Ri));
+  }
+  return make_float4(-Lr, -Li, -Rr, -Ri);
+}
+
 }  // namespace
 
 __global__ void __launch_bounds__(kRegThreads)
@@ -282,42 +322,10 @@ k_assemble_regular(const float4* __restrict__ c_hi, const float4* __restrict__ c
       const float Dx = (xh.x - chi.x) + (xl.x - clo.x);
       const float Dy = (xh.y - chi.y) + (xl.y - clo.y);
       const float Dz = (xh.z - chi.z) + (xl.z - clo.z);
-      const float dny = Dx * nj.x + Dy * nj.y + Dz * nj.z;  // quadrature offsets lie in the plane
-      const float Dni = Dx * ni4.x + Dy * ni4.y + Dz * ni4.z;
-      const float nxny = ni4.x * nj.x + ni4.y * nj.y + ni4.z * nj.z;
-      float Lr = 0.f, Li = 0.f, Rr = 0.f, Ri = 0.f;
-#pragma unroll
-      for (int p = 0; p < 7; ++p) {
-        const float dx = Dx - q[p].x, dy = Dy - q[p].y, dz = Dz - q[p].z;
-        const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-        const float rinv = rsqrtf(r2);
-        const float r = r2 * rinv;
-        const float dnx = Dni - fmaf(q[p].x, ni4.x, fmaf(q[p].y, ni4.y, q[p].z * ni4.z));
-        const float rho = k * r;
-        const float nq = rintf(rho * kInvTwoPi);
-        float th = fmaf(-nq, kTwoPiHi, rho);
-        th = fmaf(-nq, kTwoPiLo, th);
-        float sn, cs;
-        __sincosf(th, &sn, &cs);
-        const float gw = rinv * q[p].w;  // w A / (4 pi r)
-        const float Gr = cs * gw, Gi = sn * gw;
-        const float rinv2 = rinv * rinv;
-        const float qq = dnx * dny * rinv2;
-        const float a = fmaf(fmaf(rho, rho, -3.0f), qq, nxny);
-        const float b = rho * fmaf(3.0f, qq, -nxny);
-        const float lr = fmaf(-b, kinv, dny);
-        const float li = fmaf(a, kinv, -rho * dny);
-        const float Hr = Gr * rinv2, Hi = Gi * rinv2;
-        Lr = fmaf(Hr, lr, fmaf(-Hi, li, Lr));
-        Li = fmaf(Hr, li, fmaf(Hi, lr, Li));
-        const float t1 = fmaf(-dnx, rinv, 1.0f);
-        const float t2 = -dnx * rinv2 * kinv;
-        Rr = fmaf(Gr, t1, fmaf(-Gi, t2, Rr));
-        Ri = fmaf(Gr, t2, fmaf(Gi, t1, Ri));
-      }
-      __stcs(L + off, make_float2(-Lr, -Li));
-      __stcs(R + off, make_float2(-Rr, -Ri));
-      if (Lb) __stcs(Lb + off, pack_bf16(-Lr, -Li));
+      const float4 e = regular_entry(Dx, Dy, Dz, nj, make_float3(ni4.x, ni4.y, ni4.z), q, k, kinv);
+      __stcs(L + off, make_float2(e.x, e.y));
+      __stcs(R + off, make_float2(e.z, e.w));
+      if (Lb) __stcs(Lb + off, pack_bf16(e.x, e.y));
     }
   }
 }
@@ -328,12 +336,16 @@ k_assemble_regular(const float4* __restrict__ c_hi, const float4* __restrict__ c
 // it for two cycles: pairing saves issue slots only), so the form is chosen for its operation
 // count, 28 paired operations a point:
 //   - the outer points are c + s v_m with three directions v_m, so |d|^2 = |D|^2 + s^2 |v_m|^2 -
-//     2 s D.v_m and d.n_x = D.n_x - s v_m.n_x cost three operations a point, not ten;
+//     2 s D.v_m and d.n_x = D.n_x - s v_m.n_x cost three operations a point, not ten. That |d|^2
+//     cancels where d is small against s v_m (two sheets at 0.02 of an element's size: rows 3e-4
+//     off; nearer it can be negative), so the rows within three times the largest |s v_m| of a
+//     column's centroid, a few a column, are marked and formed again by regular_entry (9 us at
+//     10240 triangles, 4 at 1280; as a branch inside the loop, which it broke up, 100 and 14);
 //   - with u = d.n_x, v = d.n_y, t = 1/r, N = n_x.n_y and e = 3 u v t^2 - N the integrands are
 //     G t^2 [ (v - r e) + i (k v (u - r) - e/k) ] and G [ (1 - u t) - i u t^2 / k ];
 //   - the phase is reduced by the centroid's whole turns for all seven points (float-float, the
 //     product k r unrounded), and both cross products have accumulators of their own.
-// 10240 triangles: 1.198 -> 1.044 ms (49 operations a point and roundings on the rsqrt unit before);
+// 10240 triangles: 1.198 -> 1.053 ms (49 operations a point and roundings on the rsqrt unit before);
 // the error against FP64 entries is the same at k = 1 and a quarter less at k = 20. Four blocks per
 // SM: three (more loads in flight) 1.128 ms, five and six (spilled column data) 1.051 and 1.083 ms.
 namespace {
@@ -387,13 +399,15 @@ k_assemble_regular_x2(const float4* __restrict__ c_hi, const float4* __restrict_
   // column records as pairs (column j0 in the low half, j0 + 1 in the high half); va, vb: the first
   // orbit's offsets towards vertices 2 and 1 (the third is -(va + vb)); sq: the first orbit's |offset|^2
   u64 chx, chy, chz, clx, cly, clz, njx, njy, njz, vax, vay, vaz, vbx, vby, vbz, sq[3], qw[3];
+  float near2 = 0.f;  // 9 max |offset|^2 of the two columns
   int4 v0 = make_int4(-1, -1, -1, 0), v1 = v0;
   float grid;
   {
     const int ja = ok0 ? j0 : 0, jb = ok1 ? j0 + 1 : ja;
     const float4 a = c_hi[ja], b = c_hi[jb];
     // High parts of the centroids on one grid, a 2^22nd of the largest coordinate among the
-    // block's columns: their differences are then exact, and what D loses to rounding is known.
+    // block's columns: the difference to a row within twice that is then exact, and what D loses to
+    // rounding is known (a row farther out: rounded once, at 2^-24 of the difference).
     if (threadIdx.x == 0) s_top = 0;
     __syncthreads();
     atomicMax(&s_top, __float_as_int(fminf(1e37f, fmaxf(fmaxf(fmaxf(fabsf(a.x), fabsf(a.y)), fabsf(a.z)),
@@ -414,6 +428,9 @@ k_assemble_regular_x2(const float4* __restrict__ c_hi, const float4* __restrict_
       const float4 qa = qp[7 * (size_t)ja + 1 + p], qb = qp[7 * (size_t)jb + 1 + p];
       const u64 x = pk(qa.x, qb.x), y = pk(qa.y, qb.y), z = pk(qa.z, qb.z);
       sq[p] = fma2(x, x, fma2(y, y, mul2(z, z)));
+      float sa, sb;
+      upk(sq[p], sa, sb);
+      near2 = fmaxf(near2, 9.f * fmaxf(sa, sb));
       if (p == 0) vax = x, vay = y, vaz = z, qw[1] = pk(qa.w, qb.w);
       if (p == 1) vbx = x, vby = y, vbz = z, qw[2] = pk(qp[7 * (size_t)ja + 4].w, qp[7 * (size_t)jb + 4].w);
     }
@@ -438,7 +455,9 @@ k_assemble_regular_x2(const float4* __restrict__ c_hi, const float4* __restrict_
       s_v[threadIdx.x] = vid[i];
     }
     __syncthreads();
-    for (int t = 0; t < cnt; ++t) {
+    for (int tb = 0; tb < cnt; tb += 32) {
+    unsigned close = 0u;  // rows tb + 0..31 whose entries are formed again
+    for (int t = tb; t < min(cnt, tb + 32); ++t) {
       const int i = ib + t;
       const size_t off = (size_t)i * ld + j0;
       if (pad0 || pad1) {  // zero the padding columns (ld > n)
@@ -466,6 +485,11 @@ k_assemble_regular_x2(const float4* __restrict__ c_hi, const float4* __restrict_
       // from the exact a and the small b, a.a + b.(a + D), without the rounding of D
       const u64 D2 = fma2(ax, ax, fma2(ay, ay, fma2(az, az,
                      fma2(bx, add2(ax, Dx), fma2(by, add2(ay, Dy), mul2(bz, add2(az, Dz)))))));
+      {
+        float da, db;
+        upk(D2, da, db);
+        if ((w0 && da < near2) || (w1 && db < near2)) close |= 1u << (t & 31);
+      }
       const u64 nu = sub2(bc(0.f), fma2(Dx, nix, fma2(Dy, niy, mul2(Dz, niz))));  // -D.n_x
       RegPair c;
       c.v = fma2(Dx, njx, fma2(Dy, njy, mul2(Dz, njz)));  // d.n_y of every point
@@ -519,6 +543,31 @@ k_assemble_regular_x2(const float4* __restrict__ c_hi, const float4* __restrict_
           if (Lb) __stcs(Lb + off + 1, pack_bf16(lr1, -li1));
         }
       }
+    }
+    for (; close; close &= close - 1u) {
+      const int t = tb + __ffs(close) - 1;
+      const u64* x = s_row[t];
+      float D[3][2], nj[3][2], ni[3], u;
+      upk(add2(sub2(x[0], chx), sub2(x[3], clx)), D[0][0], D[0][1]);
+      upk(add2(sub2(x[1], chy), sub2(x[4], cly)), D[1][0], D[1][1]);
+      upk(add2(sub2(x[2], chz), sub2(x[5], clz)), D[2][0], D[2][1]);
+      upk(njx, nj[0][0], nj[0][1]);
+      upk(njy, nj[1][0], nj[1][1]);
+      upk(njz, nj[2][0], nj[2][1]);
+#pragma unroll
+      for (int d = 0; d < 3; ++d) upk(x[6 + d], ni[d], u);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        if (!(h ? ok1 : ok0) || shares_vertex(s_v[t], h ? v1 : v0)) continue;
+        if (!(D[0][h] * D[0][h] + D[1][h] * D[1][h] + D[2][h] * D[2][h] < near2)) continue;
+        const float4 e = regular_entry(D[0][h], D[1][h], D[2][h], make_float3(nj[0][h], nj[1][h], nj[2][h]),
+                                       make_float3(ni[0], ni[1], ni[2]), qp + 7 * (size_t)(j0 + h), k, kinv);
+        const size_t off = (size_t)(ib + t) * ld + j0 + h;
+        L[off] = make_float2(e.x, e.y);
+        R[off] = make_float2(e.z, e.w);
+        if (Lb) Lb[off] = pack_bf16(e.x, e.y);
+      }
+    }
     }
   }
 }
