@@ -338,14 +338,15 @@ k_assemble_regular(const float4* __restrict__ c_hi, const float4* __restrict__ c
 //   - the outer points are c + s v_m with three directions v_m, so |d|^2 = |D|^2 + s^2 |v_m|^2 -
 //     2 s D.v_m and d.n_x = D.n_x - s v_m.n_x cost three operations a point, not ten. That |d|^2
 //     cancels where d is small against s v_m (two sheets at 0.02 of an element's size: rows 3e-4
-//     off; nearer it can be negative), so the rows within three times the largest |s v_m| of a
-//     column's centroid, a few a column, are marked and formed again by regular_entry (9 us at
-//     10240 triangles, 4 at 1280; as a branch inside the loop, which it broke up, 100 and 14);
+//     off; nearer it can be negative), so the rows within sqrt(6) of the largest |s v_m| of a
+//     column's centroid, one or two a column, are marked and formed again by regular_entry (2 us at
+//     10240 triangles and at 1280; out to three times, 9 and 4 us; as a branch inside the loop,
+//     which it broke up, 100 and 14). At sqrt(6) both forms round |d|^2 at about 3 x 2^-24;
 //   - with u = d.n_x, v = d.n_y, t = 1/r, N = n_x.n_y and e = 3 u v t^2 - N the integrands are
 //     G t^2 [ (v - r e) + i (k v (u - r) - e/k) ] and G [ (1 - u t) - i u t^2 / k ];
 //   - the phase is reduced by the centroid's whole turns for all seven points (float-float, the
 //     product k r unrounded), and both cross products have accumulators of their own.
-// 10240 triangles: 1.198 -> 1.053 ms (49 operations a point and roundings on the rsqrt unit before);
+// 10240 triangles: 1.198 -> 1.046 ms (49 operations a point and roundings on the rsqrt unit before);
 // the error against FP64 entries is the same at k = 1 and a quarter less at k = 20. Four blocks per
 // SM: three (more loads in flight) 1.128 ms, five and six (spilled column data) 1.051 and 1.083 ms.
 namespace {
@@ -399,7 +400,7 @@ k_assemble_regular_x2(const float4* __restrict__ c_hi, const float4* __restrict_
   // column records as pairs (column j0 in the low half, j0 + 1 in the high half); va, vb: the first
   // orbit's offsets towards vertices 2 and 1 (the third is -(va + vb)); sq: the first orbit's |offset|^2
   u64 chx, chy, chz, clx, cly, clz, njx, njy, njz, vax, vay, vaz, vbx, vby, vbz, sq[3], qw[3];
-  float near2 = 0.f;  // 9 max |offset|^2 of the two columns
+  float near2 = 0.f;  // 6 max |offset|^2 of the two columns
   int4 v0 = make_int4(-1, -1, -1, 0), v1 = v0;
   float grid;
   {
@@ -430,7 +431,7 @@ k_assemble_regular_x2(const float4* __restrict__ c_hi, const float4* __restrict_
       sq[p] = fma2(x, x, fma2(y, y, mul2(z, z)));
       float sa, sb;
       upk(sq[p], sa, sb);
-      near2 = fmaxf(near2, 9.f * fmaxf(sa, sb));
+      near2 = fmaxf(near2, 6.f * fmaxf(sa, sb));
       if (p == 0) vax = x, vay = y, vaz = z, qw[1] = pk(qa.w, qb.w);
       if (p == 1) vbx = x, vby = y, vbz = z, qw[2] = pk(qp[7 * (size_t)ja + 4].w, qp[7 * (size_t)jb + 4].w);
     }
