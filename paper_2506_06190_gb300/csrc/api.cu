@@ -792,7 +792,7 @@ void nat_bem_destroy(nat_bem_op* op) {
   cudaStream_t s = op->stream;
   Geometry& g = op->geo;
   if (!op->geo_view) {
-    void* gp[] = {g.c_hi, g.c_lo, g.nrm, g.qp, g.vid, g.tri, g.cen, g.nrm64, g.area, g.near_pairs};
+    void* gp[] = {g.c_hi, g.c_lo, g.nrm, g.qp, g.vid, g.group, g.tri, g.cen, g.nrm64, g.area, g.near_pairs};
     for (void* p : gp) dev_free(p, s);
   }
   if (!op->views) {

@@ -158,10 +158,9 @@ nat_bem_status upload_rules(int adj_levels, int self_pts) {
 
 // ------------------------------------------------------------------------- geometry
 __global__ void k_geometry(const double* __restrict__ V, const int32_t* __restrict__ T, int n,
-                           float4* c_hi, float4* c_lo, float4* nrm, float4* qp, int4* vid,
+                           float4* c_hi, float4* c_lo, float4* nrm, float4* qp, int4* vid, float4* group,
                            double* tri, double* cen, double* nrm64, double* area) {
-  int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n) return;
+  const int at = blockIdx.x * blockDim.x + threadIdx.x, t = min(at, n - 1);
   int ia = T[3 * t], ib = T[3 * t + 1], ic = T[3 * t + 2];
   double a[3], b[3], c[3];
   for (int d = 0; d < 3; ++d) {
@@ -178,6 +177,32 @@ __global__ void k_geometry(const double* __restrict__ V, const int32_t* __restri
   double nn[3] = {cr[0] / len, cr[1] / len, cr[2] / len};
   double cc[3];
   for (int d = 0; d < 3; ++d) cc[d] = (a[d] + b[d] + c[d]) / 3.0;
+  {
+    // the warp's elements: the middle of their centroids' box, its half diagonal and sqrt(6) of the
+    // largest offset of a first-orbit point, (1 - 3a) of a vertex's; FP32 rounds the centre and points
+    const float kFirst = 1.f - 3.f * (float)c_rule7[1][0];
+    float most = 0.f, half2 = 0.f, far = 0.f, mid[3];
+    for (int d = 0; d < 3; ++d) {
+      float l = (float)cc[d], h = l;
+      for (int o = 16; o > 0; o >>= 1) {
+        l = fminf(l, __shfl_xor_sync(0xffffffffu, l, o));
+        h = fmaxf(h, __shfl_xor_sync(0xffffffffu, h, o));
+      }
+      mid[d] = 0.5f * l + 0.5f * h;
+      half2 += 0.25f * (h - l) * (h - l);
+      far = fmaxf(far, fmaxf(fabsf(l), fabsf(h)));
+    }
+    for (int v = 0; v < 3; ++v) {
+      const double* x = v == 0 ? a : v == 1 ? b : c;
+      float q2 = 0.f;
+      for (int d = 0; d < 3; ++d) q2 += (float)((x[d] - cc[d]) * (x[d] - cc[d]));
+      most = fmaxf(most, q2);
+    }
+    for (int o = 16; o > 0; o >>= 1) most = fmaxf(most, __shfl_xor_sync(0xffffffffu, most, o));
+    const float rad = 1.001f * (sqrtf(half2) + 2.45f * kFirst * sqrtf(most)) + 1e-6f * far;
+    if ((threadIdx.x & 31) == 0 && at < n) group[at >> 5] = make_float4(mid[0], mid[1], mid[2], rad * rad);
+  }
+  if (at >= n) return;
   float hi[3], lo[3];
   for (int d = 0; d < 3; ++d) {
     hi[d] = (float)cc[d];
@@ -863,6 +888,7 @@ nat_bem_status geometry_build(nat_bem_op* op, const double* dV, const int32_t* d
   NB_TRY(dev_alloc_n(&g.nrm, n, s));
   NB_TRY(dev_alloc_n(&g.qp, 7 * n, s));
   NB_TRY(dev_alloc_n(&g.vid, n, s));
+  NB_TRY(dev_alloc_n(&g.group, (n + 31) / 32, s));
   NB_TRY(dev_alloc_n(&g.tri, 9 * n, s));
   NB_TRY(dev_alloc_n(&g.cen, 3 * n, s));
   NB_TRY(dev_alloc_n(&g.nrm64, 3 * n, s));
@@ -873,7 +899,7 @@ nat_bem_status geometry_build(nat_bem_op* op, const double* dV, const int32_t* d
                               cudaMemcpyHostToDevice, s));
   const int threads = 128;
   NB_LAUNCH("geometry", s, k_geometry<<<(unsigned)((n + threads - 1) / threads), threads, 0, s>>>(
-      dV, dT, (int)n, g.c_hi, g.c_lo, g.nrm, g.qp, g.vid, g.tri, g.cen, g.nrm64, g.area));
+      dV, dT, (int)n, g.c_hi, g.c_lo, g.nrm, g.qp, g.vid, g.group, g.tri, g.cen, g.nrm64, g.area));
   NB_CHECK_LAUNCH();
   return NAT_BEM_OK;
 }

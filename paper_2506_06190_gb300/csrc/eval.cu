@@ -13,7 +13,12 @@
 // and scheduler) beside the FMA pipe, so everything else is kept small:
 //   - the rule's outer points lie on the lines from the centroid to the vertices: with D the
 //     difference to the centroid, |D - q|^2 = |D|^2 + |q|^2 - 2 D.q, and three projections D.q_m
-//     (their sum is zero) serve all six; D.n is one value per element;
+//     (their sum is zero) serve all six; D.n is one value per element. That square cancels for a
+//     point close to one of them (at 0.01 of the element's size 7e-4; nearer it can be negative): an
+//     element whose centroid is within sqrt(6) of its largest |q| is left out, marked, and added
+//     after the stage from the differences to its points. Warps whose points are away from all of
+//     a stage's elements (Geometry::group) take a loop without that test: the
+//     training field below keeps its time (669 -> 670 us), points over the surface take 5-25% longer;
 //   - the phases are reduced with the centroid's number of turns, and rounding is an FMA and an add
 //     (the rounding instruction runs on the quarter-rate unit);
 //   - two elements at a time in paired FP32 instructions.
@@ -24,6 +29,7 @@
 
 #include <mutex>
 #include <string>
+#include <type_traits>
 
 #include "internal.h"
 #include "pairs.cuh"
@@ -123,7 +129,7 @@ __device__ __forceinline__ void point_terms(u64 rinv, u64 rho, u64 turns, u64 w,
 template <int NR, int NQ>
 __global__ void __launch_bounds__(kEvalThreads)
 k_eval(const float4* __restrict__ c_hi, const float4* __restrict__ c_lo,
-       const float4* __restrict__ nrm, const float4* __restrict__ qp, int n,
+       const float4* __restrict__ nrm, const float4* __restrict__ qp, const float4* __restrict__ group, int n,
        const double* __restrict__ pts, int m, double k, const float2* __restrict__ p,
        const float2* __restrict__ g, int rhs0, int nr, int elems_per_split, double2* __restrict__ part) {
   constexpr int kF = NQ == 7 ? kFields7 : kFields1;
@@ -168,33 +174,21 @@ k_eval(const float4* __restrict__ c_hi, const float4* __restrict__ c_lo,
     __syncthreads();
     stage_elements<NQ>(s_f, c_hi, c_lo, nrm, qp, jb, cnt, grid);
     stage_data<NR, kPaired>(s_d, p, g, n, jb, cnt, rhs0, nr);
+    bool near = false;
+    if constexpr (NQ == 7) {
+      const float4 c = group[jb / kElemStage];
+      float x, y, z, u;
+      upk(add2(xh[0], xl[0]), x, u);
+      upk(add2(xh[1], xl[1]), y, u);
+      upk(add2(xh[2], xl[2]), z, u);
+      x -= c.x, y -= c.y, z -= c.z;
+      near = __any_sync(0xffffffffu, ok && fmaf(x, x, fmaf(y, y, z * z)) < c.w);
+    }
     __syncthreads();
     if (!ok) continue;
-    for (int t = 0; t < (cnt + 1) / 2; ++t) {
-      const u64* f = reinterpret_cast<const u64*>(s_f[t]);
-      const u64 ax = sub2(xh[0], f[kFHi]), bx = sub2(xl[0], f[kFLo]), Dx = add2(ax, bx);
-      const u64 ay = sub2(xh[1], f[kFHi + 1]), by = sub2(xl[1], f[kFLo + 1]), Dy = add2(ay, by);
-      const u64 az = sub2(xh[2], f[kFHi + 2]), bz = sub2(xl[2], f[kFLo + 2]), Dz = add2(az, bz);
-      const u64 D2 = fma2(ax, ax, fma2(ay, ay, fma2(az, az,
-                     fma2(bx, add2(ax, Dx), fma2(by, add2(ay, Dy), mul2(bz, add2(az, Dz)))))));
-      const u64 dn = fma2(Dx, f[kFN], fma2(Dy, f[kFN + 1], mul2(Dz, f[kFN + 2])));  // d.n of every point
-      u64 Gr = bc(0.f), Gi = Gr, Fr = Gr, Fi = Gr;
-      const u64 rc = rsqrt2(D2), rho = mul2(k2, mul2(D2, rc)), turns = turns2(rho);
-      point_terms(rc, rho, turns, f[kFW], Gr, Gi, Fr, Fi);
-      if constexpr (NQ == 7) {
-        const u64 d0 = fma2(Dx, f[kFQ0], fma2(Dy, f[kFQ0 + 1], mul2(Dz, f[kFQ0 + 2])));
-        const u64 d1 = fma2(Dx, f[kFQ1], fma2(Dy, f[kFQ1 + 1], mul2(Dz, f[kFQ1 + 2])));
-        const u64 dm[3] = {d0, d1, sub2(bc(0.f), add2(d0, d1))};
-#pragma unroll
-        for (int o = 0; o < 2; ++o)
-#pragma unroll
-          for (int q = 0; q < 3; ++q) {
-            const u64 r2 = fma2(bc(o == 0 ? -2.f : -2.f * kOrbit), dm[q], add2(D2, f[kFSq + 3 * o + q]));
-            const u64 ri = rsqrt2(r2);
-            point_terms(ri, mul2(k2, mul2(r2, ri)), turns, f[kFW + 1 + o], Gr, Gi, Fr, Fi);
-          }
-      }
-      const u64 Dr = mul2(Fr, dn), Di = mul2(Fi, dn);
+    unsigned close = 0u;  // pairs left for after the loop
+    // the pair's sums of G and dG/dn times its data
+    auto add = [&](int t, u64 Gr, u64 Gi, u64 Dr, u64 Di) {
       if constexpr (kPaired) {
         const u64 nGr = sub2(bc(0.f), Gr), nGi = sub2(bc(0.f), Gi), nDi = sub2(bc(0.f), Di);
         const u64* d = reinterpret_cast<const u64*>(s_d) + 4 * t * NR;
@@ -220,6 +214,76 @@ k_eval(const float4* __restrict__ c_hi, const float4* __restrict__ c_lo,
             ai[s] = fmaf(a.x, di[h], fmaf(a.y, dr[h], fmaf(-a.z, gi[h], fmaf(-a.w, gr[h], ai[s]))));
           }
         }
+      }
+    };
+    auto pairs = [&](auto tested) {
+      constexpr bool kTest = decltype(tested)::value;
+      for (int t = 0; t < (cnt + 1) / 2; ++t) {
+        const u64* f = reinterpret_cast<const u64*>(s_f[t]);
+        const u64 ax = sub2(xh[0], f[kFHi]), bx = sub2(xl[0], f[kFLo]), Dx = add2(ax, bx);
+        const u64 ay = sub2(xh[1], f[kFHi + 1]), by = sub2(xl[1], f[kFLo + 1]), Dy = add2(ay, by);
+        const u64 az = sub2(xh[2], f[kFHi + 2]), bz = sub2(xl[2], f[kFLo + 2]), Dz = add2(az, bz);
+        // (one point per record: D itself; its rounding is not shared by other points)
+        const u64 D2 = NQ == 1 ? fma2(Dx, Dx, fma2(Dy, Dy, mul2(Dz, Dz)))
+                               : fma2(ax, ax, fma2(ay, ay, fma2(az, az,
+                                 fma2(bx, add2(ax, Dx), fma2(by, add2(ay, Dy), mul2(bz, add2(az, Dz)))))));
+        if constexpr (kTest) {
+          float d[2], q[2], far[2] = {0.f, 0.f};
+          upk(D2, d[0], d[1]);
+#pragma unroll
+          for (int e = 0; e < 3; ++e) {
+            upk(f[kFSq + e], q[0], q[1]);
+            far[0] = fmaxf(far[0], 6.f * q[0]);
+            far[1] = fmaxf(far[1], 6.f * q[1]);
+          }
+          if (d[0] < far[0] || d[1] < far[1]) {
+            close |= 1u << t;
+            continue;
+          }
+        }
+        const u64 dn = fma2(Dx, f[kFN], fma2(Dy, f[kFN + 1], mul2(Dz, f[kFN + 2])));  // d.n of every point
+        u64 Gr = bc(0.f), Gi = Gr, Fr = Gr, Fi = Gr;
+        const u64 rc = rsqrt2(D2), rho = mul2(k2, mul2(D2, rc)), turns = turns2(rho);
+        point_terms(rc, rho, turns, f[kFW], Gr, Gi, Fr, Fi);
+        if constexpr (NQ == 7) {
+          const u64 d0 = fma2(Dx, f[kFQ0], fma2(Dy, f[kFQ0 + 1], mul2(Dz, f[kFQ0 + 2])));
+          const u64 d1 = fma2(Dx, f[kFQ1], fma2(Dy, f[kFQ1 + 1], mul2(Dz, f[kFQ1 + 2])));
+          const u64 dm[3] = {d0, d1, sub2(bc(0.f), add2(d0, d1))};
+#pragma unroll
+          for (int o = 0; o < 2; ++o)
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+              const u64 r2 = fma2(bc(o == 0 ? -2.f : -2.f * kOrbit), dm[q], add2(D2, f[kFSq + 3 * o + q]));
+              const u64 ri = rsqrt2(r2);
+              point_terms(ri, mul2(k2, mul2(r2, ri)), turns, f[kFW + 1 + o], Gr, Gi, Fr, Fi);
+            }
+        }
+        add(t, Gr, Gi, mul2(Fr, dn), mul2(Fi, dn));
+      }
+    };
+    if (!near) {
+      pairs(std::false_type{});
+      continue;
+    }
+    if constexpr (NQ == 7) {
+      pairs(std::true_type{});
+      for (; close; close &= close - 1u) {
+        const int t = __ffs(close) - 1;
+        const u64* f = reinterpret_cast<const u64*>(s_f[t]);
+        const u64 Dx = add2(sub2(xh[0], f[kFHi]), sub2(xl[0], f[kFLo]));
+        const u64 Dy = add2(sub2(xh[1], f[kFHi + 1]), sub2(xl[1], f[kFLo + 1]));
+        const u64 Dz = add2(sub2(xh[2], f[kFHi + 2]), sub2(xl[2], f[kFLo + 2]));
+        const u64 dn = fma2(Dx, f[kFN], fma2(Dy, f[kFN + 1], mul2(Dz, f[kFN + 2])));
+        const float4 *qa = qp + 7 * (size_t)(jb + 2 * t), *qb = 2 * t + 1 < cnt ? qa + 7 : qa;
+        u64 Gr = bc(0.f), Gi = Gr, Fr = Gr, Fi = Gr;
+#pragma unroll 1
+        for (int q = 0; q < 7; ++q) {
+          const float4 a = qa[q], b = qb[q];
+          const u64 dx = sub2(Dx, pk(a.x, b.x)), dy = sub2(Dy, pk(a.y, b.y)), dz = sub2(Dz, pk(a.z, b.z));
+          const u64 r2 = fma2(dx, dx, fma2(dy, dy, mul2(dz, dz))), ri = rsqrt2(r2), rho = mul2(k2, mul2(r2, ri));
+          point_terms(ri, rho, turns2(rho), f[kFW + (q + 2) / 3], Gr, Gi, Fr, Fi);
+        }
+        add(t, Gr, Gi, mul2(Fr, dn), mul2(Fi, dn));
       }
     }
   }
@@ -393,12 +457,12 @@ static void eval_launch_nq(int nr, dim3 grid, cudaStream_t s, const Geometry& g,
                            const double* d_pts, int m, double k, const float2* d_p,
                            const float2* d_g, int r0, int per, double2* part) {
   switch (eval_pass_width(nr)) {
-    case 1: k_eval<1, NQ><<<grid, kEvalThreads, 0, s>>>(g.c_hi, g.c_lo, g.nrm, g.qp, n, d_pts, m, k, d_p, d_g, r0, nr, per, part); break;
-    case 2: k_eval<2, NQ><<<grid, kEvalThreads, 0, s>>>(g.c_hi, g.c_lo, g.nrm, g.qp, n, d_pts, m, k, d_p, d_g, r0, nr, per, part); break;
-    case 4: k_eval<4, NQ><<<grid, kEvalThreads, 0, s>>>(g.c_hi, g.c_lo, g.nrm, g.qp, n, d_pts, m, k, d_p, d_g, r0, nr, per, part); break;
-    case 8: k_eval<8, NQ><<<grid, kEvalThreads, 0, s>>>(g.c_hi, g.c_lo, g.nrm, g.qp, n, d_pts, m, k, d_p, d_g, r0, nr, per, part); break;
-    case 16: k_eval<16, NQ><<<grid, kEvalThreads, 0, s>>>(g.c_hi, g.c_lo, g.nrm, g.qp, n, d_pts, m, k, d_p, d_g, r0, nr, per, part); break;
-    default: k_eval<32, NQ><<<grid, kEvalThreads, 0, s>>>(g.c_hi, g.c_lo, g.nrm, g.qp, n, d_pts, m, k, d_p, d_g, r0, nr, per, part); break;
+    case 1: k_eval<1, NQ><<<grid, kEvalThreads, 0, s>>>(g.c_hi, g.c_lo, g.nrm, g.qp, g.group, n, d_pts, m, k, d_p, d_g, r0, nr, per, part); break;
+    case 2: k_eval<2, NQ><<<grid, kEvalThreads, 0, s>>>(g.c_hi, g.c_lo, g.nrm, g.qp, g.group, n, d_pts, m, k, d_p, d_g, r0, nr, per, part); break;
+    case 4: k_eval<4, NQ><<<grid, kEvalThreads, 0, s>>>(g.c_hi, g.c_lo, g.nrm, g.qp, g.group, n, d_pts, m, k, d_p, d_g, r0, nr, per, part); break;
+    case 8: k_eval<8, NQ><<<grid, kEvalThreads, 0, s>>>(g.c_hi, g.c_lo, g.nrm, g.qp, g.group, n, d_pts, m, k, d_p, d_g, r0, nr, per, part); break;
+    case 16: k_eval<16, NQ><<<grid, kEvalThreads, 0, s>>>(g.c_hi, g.c_lo, g.nrm, g.qp, g.group, n, d_pts, m, k, d_p, d_g, r0, nr, per, part); break;
+    default: k_eval<32, NQ><<<grid, kEvalThreads, 0, s>>>(g.c_hi, g.c_lo, g.nrm, g.qp, g.group, n, d_pts, m, k, d_p, d_g, r0, nr, per, part); break;
   }
 }
 

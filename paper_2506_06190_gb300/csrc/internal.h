@@ -106,6 +106,8 @@ struct Geometry {
   float4* nrm = nullptr;      // unit outward normal (x, y, z, 0)
   float4* qp = nullptr;       // 7 per element: (y_q - c, w_q A / (4 pi)); 1 per Monte-Carlo sample
   int4* vid = nullptr;        // vertex indices (a, b, c, 0)
+  float4* group = nullptr;    // 1 per 32 elements: a centre, and the square of the distance within which
+                              // a point may be close to one of them (k_eval); meshes only
   // FP64 records
   double* tri = nullptr;      // 9 per element: vertices a, b, c
   double* cen = nullptr;      // 3 per element

@@ -144,3 +144,42 @@ def test_field_and_far_field_pass_widths_and_remainders(nb, oracle_lib, n_tri, m
         assert _rel(f[:, s], ref) < 2e-5
         ref = oracle_lib.far_field(V, F, k, dirs, p[:, s], g[:, s])
         assert _rel(far[:, s], ref) < 2e-5
+
+
+# Field points over the outer quadrature points of some elements, `height` element sizes above them:
+# d = D - q comes from parts of about half an element rounded at 2^-24 and the nearest point's term
+# goes as 1/d^2, so 4 x 2^-24 / height on top of the 2e-5 of the other field tests.
+@pytest.mark.parametrize("nrhs", [1, 3, 9, 20])
+@pytest.mark.parametrize("height", [0.3, 0.1, 0.03, 0.01, 1e-3, 1e-4])
+def test_field_close_to_quadrature_points(nb, oracle_lib, height, nrhs):
+    Vs, F = S.ring_sphere(515 - 1)
+    V = S.perturbed_ellipsoid(Vs, 42)
+    k = 2.0
+    cr = np.cross(V[F[:, 1]] - V[F[:, 0]], V[F[:, 2]] - V[F[:, 0]])
+    size, nrm = np.sqrt(np.linalg.norm(cr, axis=1)), cr / np.linalg.norm(cr, axis=1)[:, None]
+    rule, _ = oracle_lib.quad_rule()
+    t = np.arange(0, len(F), 3)
+    q = 1 + np.arange(len(t)) % 6
+    pts = np.einsum("tv,tvd->td", rule[q], V[F[t]]) + height * size[t, None] * nrm[t]
+    rng = np.random.default_rng(7)
+    p, g = ((rng.normal(size=(len(F), nrhs)) + 1j * rng.normal(size=(len(F), nrhs))).astype(np.complex64)
+            for _ in range(2))
+    with nb.Operator.assemble(V, F, k) as op:
+        f = op.evaluate(pts, p, g)
+    assert np.isfinite(f).all()
+    for s in (0, nrhs - 1):
+        ref = oracle_lib.evaluate(V, F, k, pts, p[:, s], g[:, s])
+        assert _rel(f[:, s], ref) < 2e-5 + 4 * 2.0 ** -24 / height
+
+
+@pytest.mark.parametrize("height", [1e-2, 1e-5, 1e-9])
+def test_field_close_to_monte_carlo_samples(nb, oracle_lib, height):
+    Y, N, A = S.sphere_samples(900, 1.1)
+    p, g = _data(900, 1, 43)
+    pts = Y[::7] + height * N[::7]
+    with nb.Operator.assemble_mc(Y, N, A, 2.0) as op:
+        f = op.evaluate(pts, p[:, 0], g[:, 0])
+    assert np.isfinite(f).all()
+    ref = oracle_lib.mc_evaluate(Y, N, A, 2.0, pts, p[:, 0].astype(np.complex128), g[:, 0].astype(np.complex128))
+    # hi/lo differences resolve 2^-48 of the sphere; normals and weights round at 2^-24
+    assert _rel(f, ref) < 2e-5 + 4 * 2.0 ** -48 / height
