@@ -178,7 +178,7 @@ int64_t nat_bem_required_bytes(int64_t nt, int32_t nrhs, const nat_bem_opts* opt
   int64_t b = 2 * 8 * nt * ld;                                     // L and R
   if (low_copy(o)) b += 4 * nt * ld;                               // BF16 or FP16 copy of L
   if (o.prec == NAT_BEM_PREC_MIXED_FP16) b += 4 * nt;               // its row scales
-  b += nt * (7 * 16 + 5 * 16 + 9 * 8 + 7 * 8 + 8 * 14);             // geometry + near pairs
+  b += nt * (7 * 16 + 5 * 16 + 9 * 8 + 7 * 8 + 8 * 14 + 1);         // geometry + near pairs
   b += workspace_bytes(nt, nrhs, o);
   if (nrhs >= kX6MinRhs) b += 12 * nt * ld;  // three BF16 planes of L for the accurate products
   return b;
@@ -210,7 +210,8 @@ nat_bem_status build_mesh_op(const double* verts, int64_t nv, const int32_t* tri
     NB_TRY_CUDA(cudaStreamSynchronize(s));
     T = hT.data();
   }
-  NB_TRY(validate_mesh_host(V, nv, T, nt));
+  float grid = 0.f;
+  NB_TRY(validate_mesh_host(V, nv, T, nt, &grid));
   std::vector<int2> near;
   build_near_pairs(T, nv, nt, near);
   NB_TRY(ensure_rules(o.adj_subdiv_levels, o.self_theta_pts));
@@ -228,6 +229,7 @@ nat_bem_status build_mesh_op(const double* verts, int64_t nv, const int32_t* tri
   cudaGetDevice(&op->device);
   op->geo.n = nt;
   op->geo.ld = std::max<int64_t>(ld, round_up(nt, 32));
+  op->geo.grid = grid;
   op->nn = nt;
   op->ldr = op->geo.ld;
   auto fail = [&](nat_bem_status st) {
@@ -334,7 +336,7 @@ nat_bem_status nat_bem_assemble_galerkin(const double* verts, int64_t nv, const 
     NB_TRY_CUDA(cudaMemcpyAsync(hV.data(), verts, 3 * nv * sizeof(double), cudaMemcpyDefault, s));
     NB_TRY_CUDA(cudaMemcpyAsync(hT.data(), tris, 3 * nt * sizeof(int32_t), cudaMemcpyDefault, s));
     NB_TRY_CUDA(cudaStreamSynchronize(s));
-    NB_TRY(validate_mesh_host(hV.data(), nv, hT.data(), nt));
+    NB_TRY(validate_mesh_host(hV.data(), nv, hT.data(), nt, nullptr));
     {
       // every vertex must carry a P1 unknown: each one belongs to some triangle
       std::vector<char> used(nv, 0);

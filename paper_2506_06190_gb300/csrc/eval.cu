@@ -18,11 +18,11 @@
 //     element whose centroid is within sqrt(6) of its largest |q| is left out, marked, and added
 //     after the stage from the differences to its points. Warps whose points are away from all of
 //     a stage's elements (Geometry::group) take a loop without that test: the
-//     training field below keeps its time (669 -> 670 us), points over the surface take 5-25% longer;
+//     training field below keeps its time (669 -> 673 us), points over the surface take 5-25% longer;
 //   - the phases are reduced with the centroid's number of turns, and rounding is an FMA and an add
 //     (the rounding instruction runs on the quarter-rate unit);
 //   - two elements at a time in paired FP32 instructions.
-// 10,000 points x 10240 triangles: 882 us before, 667 us now (643 without the correction of |D|^2,
+// 10,000 points x 10240 triangles: 882 us before, 673 us now (643 without the correction of |D|^2,
 // whose errors against 64 bits were 1% above the earlier kernel's; with it they are 10-15% below);
 // the far field in 2048 directions 123 -> 86 us.
 #include <cuda_runtime.h>
@@ -129,31 +129,25 @@ __device__ __forceinline__ void point_terms(u64 rinv, u64 rho, u64 turns, u64 w,
 template <int NR, int NQ>
 __global__ void __launch_bounds__(kEvalThreads)
 k_eval(const float4* __restrict__ c_hi, const float4* __restrict__ c_lo,
-       const float4* __restrict__ nrm, const float4* __restrict__ qp, const float4* __restrict__ group, int n,
-       const double* __restrict__ pts, int m, double k, const float2* __restrict__ p,
+       const float4* __restrict__ nrm, const float4* __restrict__ qp, const float4* __restrict__ group, float grid,
+       int n, const double* __restrict__ pts, int m, double k, const float2* __restrict__ p,
        const float2* __restrict__ g, int rhs0, int nr, int elems_per_split, double2* __restrict__ part) {
   constexpr int kF = NQ == 7 ? kFields7 : kFields1;
   constexpr bool kPaired = NR <= 4;  // paired accumulators: twice the registers per right-hand side
   __shared__ __align__(16) float s_f[kElemStage / 2][2 * kF];
   __shared__ float4 s_d[kElemStage * NR];
-  __shared__ int s_top;
   const int qi = blockIdx.x * kEvalThreads + threadIdx.x;
   const bool ok = qi < m;
   const u64 k2 = bc((float)k);
-  // High parts of points and centroids on one grid, a 2^22nd of the block's largest coordinate:
-  // their difference a is then exact, and with the small b of the low parts |D|^2 = a.a + b.(a + D)
-  // is free of the rounding of D = a + b (else the largest error of the sum, three times the rest).
-  if (threadIdx.x == 0) s_top = 0;
-  __syncthreads();
+  if (NQ == 1) grid = 0.f;
+  // High parts of points and centroids on the body's grid: their difference a is exact out to a few
+  // diameters of the body, and with the small b of the low parts |D|^2 = a.a + b.(a + D) is free of
+  // the rounding of D = a + b (else the largest error of the sum, three times the rest). Beyond, a
+  // rounds at 2^-24. Nothing here depends on the call's other points. One-point records split where
+  // FP32 does (grid 0) and square D: no other point shares its rounding.
   double v[3];
 #pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    v[d] = ok ? pts[3 * (size_t)qi + d] : 0.0;
-    const float a = fabsf((float)v[d]);
-    if (a < 1e37f) atomicMax(&s_top, __float_as_int(a));
-  }
-  __syncthreads();
-  const float grid = 3.f * __int_as_float((s_top & 0x7f800000) + 0x00800000);
+  for (int d = 0; d < 3; ++d) v[d] = ok ? pts[3 * (size_t)qi + d] : 0.0;
   u64 xh[3], xl[3];
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
@@ -223,7 +217,6 @@ k_eval(const float4* __restrict__ c_hi, const float4* __restrict__ c_lo,
         const u64 ax = sub2(xh[0], f[kFHi]), bx = sub2(xl[0], f[kFLo]), Dx = add2(ax, bx);
         const u64 ay = sub2(xh[1], f[kFHi + 1]), by = sub2(xl[1], f[kFLo + 1]), Dy = add2(ay, by);
         const u64 az = sub2(xh[2], f[kFHi + 2]), bz = sub2(xl[2], f[kFLo + 2]), Dz = add2(az, bz);
-        // (one point per record: D itself; its rounding is not shared by other points)
         const u64 D2 = NQ == 1 ? fma2(Dx, Dx, fma2(Dy, Dy, mul2(Dz, Dz)))
                                : fma2(ax, ax, fma2(ay, ay, fma2(az, az,
                                  fma2(bx, add2(ax, Dx), fma2(by, add2(ay, Dy), mul2(bz, add2(az, Dz)))))));
@@ -457,12 +450,12 @@ static void eval_launch_nq(int nr, dim3 grid, cudaStream_t s, const Geometry& g,
                            const double* d_pts, int m, double k, const float2* d_p,
                            const float2* d_g, int r0, int per, double2* part) {
   switch (eval_pass_width(nr)) {
-    case 1: k_eval<1, NQ><<<grid, kEvalThreads, 0, s>>>(g.c_hi, g.c_lo, g.nrm, g.qp, g.group, n, d_pts, m, k, d_p, d_g, r0, nr, per, part); break;
-    case 2: k_eval<2, NQ><<<grid, kEvalThreads, 0, s>>>(g.c_hi, g.c_lo, g.nrm, g.qp, g.group, n, d_pts, m, k, d_p, d_g, r0, nr, per, part); break;
-    case 4: k_eval<4, NQ><<<grid, kEvalThreads, 0, s>>>(g.c_hi, g.c_lo, g.nrm, g.qp, g.group, n, d_pts, m, k, d_p, d_g, r0, nr, per, part); break;
-    case 8: k_eval<8, NQ><<<grid, kEvalThreads, 0, s>>>(g.c_hi, g.c_lo, g.nrm, g.qp, g.group, n, d_pts, m, k, d_p, d_g, r0, nr, per, part); break;
-    case 16: k_eval<16, NQ><<<grid, kEvalThreads, 0, s>>>(g.c_hi, g.c_lo, g.nrm, g.qp, g.group, n, d_pts, m, k, d_p, d_g, r0, nr, per, part); break;
-    default: k_eval<32, NQ><<<grid, kEvalThreads, 0, s>>>(g.c_hi, g.c_lo, g.nrm, g.qp, g.group, n, d_pts, m, k, d_p, d_g, r0, nr, per, part); break;
+    case 1: k_eval<1, NQ><<<grid, kEvalThreads, 0, s>>>(g.c_hi, g.c_lo, g.nrm, g.qp, g.group, g.grid, n, d_pts, m, k, d_p, d_g, r0, nr, per, part); break;
+    case 2: k_eval<2, NQ><<<grid, kEvalThreads, 0, s>>>(g.c_hi, g.c_lo, g.nrm, g.qp, g.group, g.grid, n, d_pts, m, k, d_p, d_g, r0, nr, per, part); break;
+    case 4: k_eval<4, NQ><<<grid, kEvalThreads, 0, s>>>(g.c_hi, g.c_lo, g.nrm, g.qp, g.group, g.grid, n, d_pts, m, k, d_p, d_g, r0, nr, per, part); break;
+    case 8: k_eval<8, NQ><<<grid, kEvalThreads, 0, s>>>(g.c_hi, g.c_lo, g.nrm, g.qp, g.group, g.grid, n, d_pts, m, k, d_p, d_g, r0, nr, per, part); break;
+    case 16: k_eval<16, NQ><<<grid, kEvalThreads, 0, s>>>(g.c_hi, g.c_lo, g.nrm, g.qp, g.group, g.grid, n, d_pts, m, k, d_p, d_g, r0, nr, per, part); break;
+    default: k_eval<32, NQ><<<grid, kEvalThreads, 0, s>>>(g.c_hi, g.c_lo, g.nrm, g.qp, g.group, g.grid, n, d_pts, m, k, d_p, d_g, r0, nr, per, part); break;
   }
 }
 

@@ -105,6 +105,7 @@ struct Geometry {
   float4* c_lo = nullptr;     // centroid, low part: c = hi + lo to ~2^-48 relative
   float4* nrm = nullptr;      // unit outward normal (x, y, z, 0)
   float4* qp = nullptr;       // 7 per element: (y_q - c, w_q A / (4 pi)); 1 per Monte-Carlo sample
+  float grid = 0.f;           // meshes: k_eval's spacing of high parts (split_grid)
   int4* vid = nullptr;        // vertex indices (a, b, c, 0)
   float4* group = nullptr;    // 1 per 32 elements: a centre, and the square of the distance within which
                               // a point may be close to one of them (k_eval); meshes only
@@ -129,7 +130,12 @@ struct Galerkin {
 
 // Host-side mesh check and near-pair list (mesh.cpp). Returns NAT_BEM_EINVAL with a message
 // for an invalid mesh.
-nat_bem_status validate_mesh_host(const double* V, int64_t nv, const int32_t* T, int64_t nt);
+// grid, unless null: split_grid of its triangles' box.
+nat_bem_status validate_mesh_host(const double* V, int64_t nv, const int32_t* T, int64_t nt, float* grid);
+// For a body in the box lo..hi: three times a power of two such that (x + grid) - grid rounds the
+// coordinates of points within about four diameters of it to one spacing, fine enough for their
+// differences to be exact in FP32. Farther points round by themselves, to their own FP32 spacing.
+float split_grid(const double* lo, const double* hi);
 void build_near_pairs(const int32_t* T, int64_t nv, int64_t nt, std::vector<int2>& pairs);
 
 // Quadrature tables the kernels read from constant memory (assemble.cu).

@@ -24,7 +24,16 @@ double vdot(V3 a, V3 b) { return a.x * b.x + a.y * b.y + a.z * b.z; }
 
 }  // namespace
 
-nat_bem_status validate_mesh_host(const double* V, int64_t nv, const int32_t* T, int64_t nt) {
+float split_grid(const double* lo, const double* hi) {
+  double reach = 0.0;
+  for (int d = 0; d < 3; ++d)
+    reach = std::max(reach, std::max(std::fabs(lo[d]), std::fabs(hi[d])) + 4.0 * (hi[d] - lo[d]));
+  int e = 0;
+  std::frexp(std::min(std::max(reach, 1e-36), 1e36), &e);  // reach < 2^e
+  return std::ldexp(3.f, e);
+}
+
+nat_bem_status validate_mesh_host(const double* V, int64_t nv, const int32_t* T, int64_t nt, float* grid) {
   if (nv <= 0 || nt <= 0) {
     set_error("mesh: need nv > 0 and nt > 0");
     return NAT_BEM_EINVAL;
@@ -88,6 +97,15 @@ nat_bem_status validate_mesh_host(const double* V, int64_t nv, const int32_t* T,
     set_error("mesh: enclosed volume is not positive (inward winding)");
     return NAT_BEM_EINVAL;
   }
+  if (!grid) return NAT_BEM_OK;
+  double lo[3] = {HUGE_VAL, HUGE_VAL, HUGE_VAL}, hi[3] = {-HUGE_VAL, -HUGE_VAL, -HUGE_VAL};
+  for (int64_t v = 0; v < nv; ++v)
+    if (first[v + 1] > first[v])  // the triangles' vertices
+      for (int d = 0; d < 3; ++d) {
+        lo[d] = std::min(lo[d], V[3 * v + d]);
+        hi[d] = std::max(hi[d], V[3 * v + d]);
+      }
+  *grid = split_grid(lo, hi);
   return NAT_BEM_OK;
 }
 

@@ -183,3 +183,20 @@ def test_field_close_to_monte_carlo_samples(nb, oracle_lib, height):
     ref = oracle_lib.mc_evaluate(Y, N, A, 2.0, pts, p[:, 0].astype(np.complex128), g[:, 0].astype(np.complex128))
     # hi/lo differences resolve 2^-48 of the sphere; normals and weights round at 2^-24
     assert _rel(f, ref) < 2e-5 + 4 * 2.0 ** -48 / height
+
+
+@pytest.mark.parametrize("shift", [0.0, 500.0])
+def test_a_point_does_not_depend_on_the_others(nb, oracle_lib, shift):
+    """The same points beside one at 1e30, which once took the low parts of the others' coordinates."""
+    Vs, F = S.ring_sphere(600)
+    V = S.perturbed_ellipsoid(Vs, 44) + shift
+    k = 2.0
+    p, g = _data(len(F), 1, 45)
+    pts = S.shell_points(128, 1.5, 6.0, 4) + shift
+    far = pts.copy()
+    far[-1] = 1e30
+    with nb.Operator.assemble(V, F, k) as op:
+        a, b = op.evaluate(pts, p[:, 0], g[:, 0]), op.evaluate(far, p[:, 0], g[:, 0])
+    assert np.array_equal(a[:-1], b[:-1])
+    ref = oracle_lib.evaluate(V, F, k, pts, p[:, 0].astype(np.complex128), g[:, 0].astype(np.complex128))
+    assert _rel(a, ref) < 2e-5  # as in test_field_and_far_field_pass_widths_and_remainders
