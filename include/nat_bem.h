@@ -203,7 +203,7 @@ NAT_BEM_API nat_bem_status nat_bem_assemble_mc(const double* pts, const double* 
  * NAT_BEM_EINVAL: NULL arrays, nv or nt < 1, m < 0 or > 2^31 - 1, radius not positive and
  * finite, a triangle index out of range, a degenerate triangle, more than 2^28 grid cells,
  * more samples than cap. NAT_BEM_ENOMEM / NAT_BEM_ECUDA as for nat_bem_assemble.
- * NAT_BEM_ETIMEOUT: a bounded wait between phases gave up.
+ * NAT_BEM_ETIMEOUT: the device made no progress for two seconds.
  */
 NAT_BEM_API nat_bem_status nat_bem_poisson_sample(const double* verts, int64_t nv, const int32_t* tris,
                                                   int64_t nt, double radius, const double* u, int64_t m,

@@ -62,7 +62,7 @@ struct PsInfo {
   unsigned bar;                     // grid barrier arrivals
   int err;                          // a bounded wait gave up
   int count;                        // accepted samples
-  unsigned pad;
+  unsigned beat;                    // batches of candidates looked at in long lists
   unsigned done[kPsStripes][32];    // cells decided, counted on several cache lines
 };
 
@@ -215,13 +215,14 @@ __device__ __forceinline__ unsigned ps_load(const unsigned* p) {
 __device__ __forceinline__ void ps_count(unsigned* p) {
   asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p) : "memory");
 }
-// One thread: waits until *p >= target, at most two seconds (then the error word is set).
+// Whether two seconds have passed since t0 (0: from now on).
 __device__ __forceinline__ bool ps_late(uint64_t& t0) {
   uint64_t t;
   asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
   if (t0 == 0) t0 = t;
   return t - t0 > 2000000000ull;
 }
+// One thread: waits until *p >= target, at most two seconds (then the error word is set).
 __device__ __forceinline__ bool ps_wait(const unsigned* p, unsigned target, int* err) {
   uint64_t t0 = 0;
   for (unsigned it = 1;; ++it) {
@@ -281,17 +282,24 @@ k_ps_run(PsGrid g, double r2, const double* __restrict__ V, const int32_t* __res
   }
   if (!barrier((unsigned)G)) return;
   if (w == kPsWorkers) {
-    // the counters' sum for the block's warps, until every cell is decided
+    // the counters' sum for the block's warps, until every cell is decided; gives up when for two
+    // seconds no cell was decided and no long list advanced
     uint64_t t0 = 0;
+    unsigned seen = 0u;
     for (unsigned it = 1; s_done < n && !s_bad; ++it) {
       unsigned v = lane < kPsStripes ? ps_load(&info->done[lane][0]) : 0u;
       v = __reduce_add_sync(0xffffffffu, v);
       if (lane == 0) {
         __threadfence_block();
         s_done = (int)v;
-        if ((it & 255u) == 0u && ps_late(t0)) {
-          atomicOr(&info->err, 1);
-          s_bad = 1;
+        if ((it & 255u) == 0u) {
+          const unsigned now = v + ps_load(&info->beat);
+          if (now != seen) t0 = 0;
+          seen = now;
+          if (ps_late(t0)) {
+            atomicOr(&info->err, 1);
+            s_bad = 1;
+          }
         }
       }
       __syncwarp();
@@ -349,7 +357,8 @@ k_ps_run(PsGrid g, double r2, const double* __restrict__ V, const int32_t* __res
     }
     int best = -1;
     float4 bh = mh, bl = ml;
-    while (cnt > 0) {
+    for (unsigned batch = 1; cnt > 0; ++batch) {
+      if ((batch & 31u) == 0u && lane == 0) ps_count(&info->beat);
       for (int c = 0; c < cnt; ++c) {
         const int ci = __shfl_sync(0xffffffffu, mine, c);
         if (best >= 0 && ci > best) continue;

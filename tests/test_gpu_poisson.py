@@ -135,3 +135,13 @@ def test_distances_at_the_radius(nb, scale, shift):
     for r in np.sort(d)[[5, 40, 120]]:
         for q in (r, np.nextafter(r, 0.0), np.nextafter(r, 1e300)):
             _check(nb, V, F, u, float(q))
+
+
+def test_seconds_of_work_in_one_cell(nb):
+    """A radius beyond the body's size puts every draw into one cell, whose list one warp walks: a few
+    seconds at this many draws, with no cell decided meanwhile. The lowest draw is accepted."""
+    V, F = S.octahedron()
+    u = np.tile(np.random.default_rng(11).random((1_000_000, 3)), (20, 1))
+    idx, x, n = nb.nat_bem_poisson_sample(V, F, u, 50.0, cap=16)
+    ai, ax, an = P.sample(V, F, u[:1], 50.0)
+    assert list(idx) == [0] and np.array_equal(x, ax) and np.array_equal(n, an)
