@@ -212,6 +212,11 @@ __device__ __forceinline__ unsigned ps_load(const unsigned* p) {
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
 }
+__device__ __forceinline__ unsigned ps_peek(const unsigned* p) {
+  unsigned v;
+  asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
 __device__ __forceinline__ void ps_count(unsigned* p) {
   asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p) : "memory");
 }
@@ -285,15 +290,22 @@ k_ps_run(PsGrid g, double r2, const double* __restrict__ V, const int32_t* __res
     // the counters' sum for the block's warps, until every cell is decided; gives up when for two
     // seconds no cell was decided and no long list advanced
     uint64_t t0 = 0;
-    unsigned seen = 0u;
+    unsigned seen = 0u, last = 0u, still = 0u;
     for (unsigned it = 1; s_done < n && !s_bad; ++it) {
-      unsigned v = lane < kPsStripes ? ps_load(&info->done[lane][0]) : 0u;
+      // An acquiring load empties the SM's L1, which a warp on a long list walks from (172 ns a
+      // candidate, 64 without): after a while without news the polls are relaxed ones, and a fence
+      // acquires what they find.
+      const bool quiet = still >= 64u;
+      unsigned v = lane >= kPsStripes ? 0u : quiet ? ps_peek(&info->done[lane][0]) : ps_load(&info->done[lane][0]);
       v = __reduce_add_sync(0xffffffffu, v);
+      if (quiet && v != last) __threadfence();
+      still = v == last ? still + 1u : 0u;
+      last = v;
       if (lane == 0) {
         __threadfence_block();
         s_done = (int)v;
         if ((it & 255u) == 0u) {
-          const unsigned now = v + ps_load(&info->beat);
+          const unsigned now = v + ps_peek(&info->beat);
           if (now != seen) t0 = 0;
           seen = now;
           if (ps_late(t0)) {
@@ -359,9 +371,12 @@ k_ps_run(PsGrid g, double r2, const double* __restrict__ V, const int32_t* __res
     float4 bh = mh, bl = ml;
     for (unsigned batch = 1; cnt > 0; ++batch) {
       if ((batch & 31u) == 0u && lane == 0) ps_count(&info->beat);
-      for (int c = 0; c < cnt; ++c) {
+      // the candidates below the best one yet, in list order
+      unsigned todo = __ballot_sync(0xffffffffu, mine >= 0 && (best < 0 || mine < best));
+      while (todo) {
+        const int c = __ffs(todo) - 1;
+        todo &= todo - 1u;
         const int ci = __shfl_sync(0xffffffffu, mine, c);
-        if (best >= 0 && ci > best) continue;
         const float hx = __shfl_sync(0xffffffffu, mh.x, c), hy = __shfl_sync(0xffffffffu, mh.y, c),
                     hz = __shfl_sync(0xffffffffu, mh.z, c);
         const float lx = __shfl_sync(0xffffffffu, ml.x, c), ly = __shfl_sync(0xffffffffu, ml.y, c),
@@ -392,13 +407,14 @@ k_ps_run(PsGrid g, double r2, const double* __restrict__ V, const int32_t* __res
         best = ci;
         bh = make_float4(hx, hy, hz, __int_as_float(ci));
         bl = make_float4(lx, ly, lz, 0.f);
+        todo &= __ballot_sync(0xffffffffu, mine < best);
       }
       mine = -1;  // the next 32 of a longer list
       for (cnt = 0; cnt < 32 && nxt >= 0; ++cnt) {
         if (lane == cnt) mine = nxt;
         nxt = next[nxt];
       }
-      if (mine >= 0) {
+      if (mine >= 0 && (best < 0 || mine < best)) {
         mh = hi4[mine];
         ml = lo4[mine];
       }
