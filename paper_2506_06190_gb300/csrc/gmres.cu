@@ -58,7 +58,7 @@ struct Workspace {
   unsigned* gbar = nullptr;                                // grid barrier state (count, gen)
   int coop_blocks = 0;                                     // 0: fused kernel not usable
   int units_blocks = 0;                                    // grid of the multi-RHS fused kernel
-  bool run_ok = false;                                     // one RHS: whole runs by k_gmres_run
+  bool run_ok = false;                                     // k_gmres_run usable (one RHS, or a batch)
   double2 *pblk = nullptr, *hred = nullptr;                // fused kernel: block partials, totals
   int arn_smem = 0;                                        // fused kernel: dynamic shared bytes
   double2* pbu = nullptr;                                  // multi-RHS fused kernel: unit partials
@@ -2198,7 +2198,7 @@ static nat_bem_status workspace_ensure(nat_bem_op* op, int nrhs, cudaStream_t s)
         take(&ws->dec, nr);
       }
       take(&ws->wf, (size_t)n * nr);  // FP32 w of inner solves on the FP32 basis
-      ws->run_ok = (nrhs == 1 || op->bstride > 0) && !std::getenv("NATBEM_NO_RUN_KERNEL") && run_usable();
+      ws->run_ok = !std::getenv("NATBEM_NO_RUN_KERNEL") && run_usable();
     }
   }
   char* tc = nullptr;
@@ -2621,7 +2621,8 @@ static nat_bem_status gmres_run(nat_bem_op* op, Workspace* ws, const GArgs& a, i
   // times). Measured with one solve in flight, two-launch form -> this, a whole solve: 1280 rows
   // FP32 1037 -> 478 us, 3956 783 -> 466, 5174 1888 -> 1401, 10240 5878 -> 4299; 10240 mixed BF16
   // 4283 -> 3643. Above that the matvec streams for 10x the time of the rest of an iteration.
-  if (ws->run_ok && (engine == kEngineGemv || engine == kEngineGemvCopy) && !tracing_enabled()) {
+  if (ws->run_ok && (nrhs == 1 || op->bstride > 0) && (engine == kEngineGemv || engine == kEngineGemvCopy) &&
+      !tracing_enabled()) {
     const int fmt = engine == kEngineGemv ? 0 : (op->copy_fp16 ? 2 : 1);
     int at_once = 1;
     const RunArgs shape = run_fit(n, (int)ws->ld, ws->coop_blocks, nrhs, std::max(1, op->share), fmt, a.Vf != nullptr,

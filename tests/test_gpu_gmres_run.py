@@ -111,3 +111,18 @@ def test_mixed_solves_end_well_below_the_tolerance(nb, oracle_lib, prec):
             L, R = oracle_lib.assemble(job["V"], job["F"], job["k"])
             ref = np.linalg.solve(L, R @ job["neumann"].astype(np.complex128))
             assert max(_rel(x, ref), _rel(r[0], ref)) < 1e-6
+
+
+@pytest.mark.parametrize("prec", ["fp32", "bf16"])
+def test_single_solve_after_several_right_hand_sides(nb, prec):
+    """A workspace made for several right-hand sides serves one as a fresh one does: the same bits."""
+    Vs, F = S.ring_sphere(1218)
+    V = S.perturbed_ellipsoid(Vs, 71)
+    g = S.monopole_neumann(V, F, 3.0).astype(np.complex64)
+    opts = nb.nat_bem_opts_default(prec={"fp32": nb.PREC_FP32, "bf16": nb.PREC_MIXED_BF16}[prec])
+    with nb.Operator.assemble(V, F, 3.0, opts) as op:
+        fresh, a, _ = op.solve(g)
+    with nb.Operator.assemble(V, F, 3.0, opts) as op:
+        op.solve(np.asfortranarray(np.stack([g, 2 * g, 1j * g, g, -g, g], 1)))
+        x, b, st = op.solve(g)
+    assert st == nb.NAT_BEM_OK and a.iterations == b.iterations and np.array_equal(x, fresh)
