@@ -57,7 +57,7 @@ struct Workspace {
   int* outer_done = nullptr;                               // refinement: converged RHS
   unsigned* gbar = nullptr;                                // grid barrier state (count, gen)
   int coop_blocks = 0;                                     // 0: fused kernel not usable
-  int units_blocks = 0;                                    // grid of the multi-RHS fused kernel
+  int units_sms = 0, units_most = 0;                       // multi-RHS fused kernel: SMs, blocks that fit on one
   bool run_ok = false;                                     // k_gmres_run usable (one RHS, or a batch)
   double2 *pblk = nullptr, *hred = nullptr;                // fused kernel: block partials, totals
   int arn_smem = 0;                                        // fused kernel: dynamic shared bytes
@@ -943,9 +943,11 @@ constexpr int kArnPanelBytesF32 = 48 * 1024;
 constexpr int kArnMaxRhs = 256;
 constexpr int kArnUnitsMinRhs = 4;  // more right-hand sides than this: k_arnoldi_units
 // k_arnoldi_units: blocks per SM (at most). Three keep more loads in flight where the basis streams
-// from memory (20480 rows x 64 RHS: 82 -> 70 us a step); with small systems, several of which run
-// side by side in a batch, a grid that leaves room for the others' blocks does better (six
-// requests of up to 6k rows x 48 RHS: 36 ms with two, 43 ms with three).
+// from memory: a solve by itself takes 1 to 4% less from 5174 rows x 64 RHS up (12000 x 64: 16.7 ->
+// 15.9 ms; 20480 x 64: 44.8 -> 43.5, 82 -> 70 us a step), nothing below. But the solves of a batch run
+// side by side, and there a grid that leaves room for the others' blocks does better: six requests of
+// 1000 to 16000 rows x 1 to 32 RHS take 36.5 ms with two and 42.8 ms with three. A call cannot see
+// its neighbours, so the line lies above what batches hold.
 constexpr int arn_units_per_sm(int64_t n, int64_t nrhs) { return n * nrhs >= (1 << 20) ? 3 : 2; }
 // mixed refinement: a stalled sweep with every open true residual within this factor of the
 // tolerance ends the solve (the FP32 residual product's rounding floor)
@@ -2091,6 +2093,11 @@ void workspace_free(Workspace* ws, cudaStream_t s) {
   delete ws;
 }
 
+// Blocks of k_arnoldi_units for nrhs right-hand sides: the solve's own number, not the workspace's.
+static int units_grid(const Workspace* ws, int64_t n, int nrhs) {
+  return ws->units_sms * std::min(arn_units_per_sm(n, nrhs), ws->units_most);
+}
+
 static nat_bem_status workspace_ensure(nat_bem_op* op, int nrhs, cudaStream_t s) {
   const int m = krylov_dim(op->opts);
   Workspace* ws = op->ws;
@@ -2188,10 +2195,11 @@ static nat_bem_status workspace_ensure(nat_bem_op* op, int nrhs, cudaStream_t s)
         int pu32 = 0, pu64 = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pu32, k_arnoldi_units<true>, 256, 0);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pu64, k_arnoldi_units<false>, 256, 0);
-        ws->units_blocks = sms * std::max(1, std::min(arn_units_per_sm(n, nrhs), std::min(pu32, pu64)));
+        ws->units_sms = sms;
+        ws->units_most = std::max(1, std::min(pu32, pu64));
         size_t most = 0;
         for (int q = kArnUnitsMinRhs + 1; q <= nrhs; ++q) {
-          const int u = arnoldi_unit((int)n, q, ws->units_blocks);
+          const int u = arnoldi_unit((int)n, q, units_grid(ws, n, q));
           most = std::max(most, (size_t)q * (size_t)((n + u - 1) / u));
         }
         take(&ws->pbu, most * (mm + 2));
@@ -2680,11 +2688,12 @@ static nat_bem_status gmres_run(nat_bem_op* op, Workspace* ws, const GArgs& a, i
         int* errp = ws->tc_err;
         if (nrhs > kArnUnitsMinRhs && ws->pbu) {
           double2 *pu = ws->pbu, *dec = ws->dec;
-          int unit = arnoldi_unit(n, nrhs, ws->units_blocks);
+          const int grid = units_grid(ws, n, nrhs);
+          int unit = arnoldi_unit(n, nrhs, grid);
           int cps = (n + unit - 1) / unit, w32 = yf != nullptr;
           void* args[] = {&ac, &pu, &hr, &dec, &bar, &errp, &unit, &cps, &w32};
           const void* kern = ac.Vf ? (const void*)k_arnoldi_units<true> : (const void*)k_arnoldi_units<false>;
-          NB_LAUNCH("gmres_arnoldi", s, NB_TRY_CUDA(cudaLaunchCooperativeKernel(kern, dim3(ws->units_blocks), dim3(256), args, 0, s)));
+          NB_LAUNCH("gmres_arnoldi", s, NB_TRY_CUDA(cudaLaunchCooperativeKernel(kern, dim3(grid), dim3(256), args, 0, s)));
           continue;
         }
         const int smem = ac.Vf ? std::min(ws->arn_smem, kArnPanelBytesF32) : ws->arn_smem;

@@ -73,3 +73,20 @@ def test_right_hand_sides_through_the_split_of_r(nb, m):
                 b = R @ h
                 res = np.linalg.norm(L @ np.asarray(x) - b, axis=0)
                 assert np.max(res - 5e-6 * np.linalg.norm(b, axis=0)) <= 0
+
+
+def test_fewer_right_hand_sides_after_many(nb):
+    """A workspace made for many right-hand sides (n nrhs above 2^20: a larger grid for the Arnoldi
+    step) gives fewer of them the bits of a fresh one."""
+    Vs, F = S.ring_sphere(5174)
+    V = S.perturbed_ellipsoid(Vs, 72)
+    rng = np.random.default_rng(73)
+    g = (rng.normal(size=(len(F), 208)) + 1j * rng.normal(size=(len(F), 208))).astype(np.complex64)
+    few = np.asfortranarray(g[:, :64])
+    opts = nb.nat_bem_opts_default(max_iter=80)
+    with nb.Operator.assemble(V, F, 2.0, opts) as op:
+        fresh, a, _ = op.solve(few)
+    with nb.Operator.assemble(V, F, 2.0, opts) as op:
+        op.solve(np.asfortranarray(g))
+        x, b, st = op.solve(few)
+    assert st == nb.NAT_BEM_OK and a.iterations == b.iterations and np.array_equal(x, fresh)
