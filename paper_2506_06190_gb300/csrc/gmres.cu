@@ -3090,7 +3090,7 @@ nat_bem_status solve_impl(nat_bem_op* op, const float2* d_neumann, int nrhs, flo
     }
   }
   if (tc_err) {
-    set_error("tensor-core product: a bounded wait gave up (code " + std::to_string(tc_err) + ")");
+    set_error("GMRES: a bounded wait gave up (code " + std::to_string(tc_err) + ")");
     return NAT_BEM_ECUDA;
   }
   int maxit = 0;

@@ -640,7 +640,7 @@ extern "C" nat_bem_status nat_bem_poisson_sample(const double* verts, int64_t nv
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_failed(e);
     if (h.err) {
-      set_error("nat_bem_poisson_sample: a bounded wait gave up");
+      set_error("nat_bem_poisson_sample: no progress for two seconds");
       return failed(NAT_BEM_ETIMEOUT);
     }
     *count = h.count;
