@@ -958,13 +958,14 @@ constexpr double kResidualFloor = 4.0;
 // adds 0.4e-2 of a sweep's start to its end, so tighter ones gain little).
 // Ten bodies of 10240 triangles: 371 iterations in 40 sweeps and errors up to 0.57e-6, against 372 in
 // 39 and up to 1.0e-6 when a sweep was only ever loosened, in whole octaves, towards 0.7 tol; 240
-// solves in buckets of 500 to 8000 triangles: 9224 in 1014 and up to 0.89e-6, against 9094 in 940
-// and up to 1.14e-6 (the batch of 24 takes 2% longer).
+// solves in buckets of 500 to 8000 triangles: 9187 in 952 and up to 0.90e-6, against 9094 in 940
+// and up to 1.14e-6 (the batch of 24 takes 2% longer). 64 wavenumbers of one body, many of them with a
+// floor near tol: 4408 in 260, against 4404 in 256 (145.6-147.0 solves/s, four in flight, and 146.4-146.6).
 constexpr double kSweepTarget = 0.6;
 // A residual is left alone below this part of tol. Above it, and below tol, another sweep of an
-// iteration or two follows (several right-hand sides: while one is above tol), unless they have
-// stopped contracting: where a sweep ends just under tol or just over it is decided by rounding,
-// and with it whether a solution ends 1.1e-6 or 0.2e-6 off.
+// iteration or two follows (several right-hand sides: while one is above tol), unless it is the floor
+// that the sweep has reached: where a sweep ends just under tol or just over it is decided by
+// rounding, and with it whether a solution ends 1.1e-6 or 0.2e-6 off.
 constexpr double kSweepLeave = 0.75;
 
 // The inner tolerance of the next refinement sweep when the largest open relative residual is
@@ -3023,8 +3024,7 @@ nat_bem_status solve_impl(nat_bem_op* op, const float2* d_neumann, int nrhs, flo
       const bool fp32_basis =
           !fp64_basis && ws->coop_blocks > 0 && ws->wf && (nrhs <= kArnUnitsMinRhs || ws->pbu != nullptr);
       // The last sweeps need only the contraction still missing to the outer target
-      // (sweep_inner_tol); NATBEM_FIXED_INNER_TOL keeps
-      // inner_tol for every sweep.
+      // (sweep_inner_tol); NATBEM_FIXED_INNER_TOL keeps inner_tol for every sweep.
       static const bool fixed_inner = std::getenv("NATBEM_FIXED_INNER_TOL") != nullptr;
       for (int sweep = 0; sweep < o.max_refinements && budget > 0; ++sweep) {
         double rho = 0.0;
@@ -3035,9 +3035,11 @@ nat_bem_status solve_impl(nat_bem_op* op, const float2* d_neumann, int nrhs, flo
         a.Vf = fp32_basis ? reinterpret_cast<float2*>(ws->V) : nullptr;
         NB_TRY(sweep_once(inner, kSweepLeave * o.tol));
         a.Vf = nullptr;
-        bool left = true;  // every right-hand side is below kSweepLeave x tol
-        for (int q = 0; q < nrhs; ++q) left = left && od[q];
-        if (left || (converged && !gemv_path)) break;
+        // below tol, but not below kSweepLeave x tol: worth another sweep where the residual is what
+        // the sweep was asked for, not the floor
+        bool more = false;
+        for (int q = 0; q < nrhs; ++q) more = more || (!od[q] && rt[q] <= 1.25 * a.tol * prev[q]);
+        if (converged && !(gemv_path && more)) break;
         // A sweep that shrank some residual by less than 10x (the low-precision operator's
         // error is comparable to the inner tolerance: high k, ill-conditioned L) or that used
         // up the budget: the rest is solved with the FP32 operator below, with a fresh
@@ -3052,11 +3054,11 @@ nat_bem_status solve_impl(nat_bem_op* op, const float2* d_neumann, int nrhs, flo
         double worst = 0.0;
         bool at_floor = true;
         for (int q = 0; q < nrhs; ++q)
-          if (!(converged ? od[q] : conv[q])) {
+          if (!conv[q]) {
             worst = std::max(worst, rt[q] / prev[q]);
             at_floor = at_floor && rt[q] <= kResidualFloor * o.tol;
           }
-        if (converged && (worst > stall || budget <= 0)) break;
+        if (converged && budget <= 0) break;
         if (worst > stall && at_floor) {
           converged = true;
           for (int q = 0; q < nrhs; ++q) conv[q] = 1;
